@@ -109,7 +109,7 @@ def measured_peaks():
 
 
 # Sources of the draft-attention call (the kernels whose DRAM traffic profiles/traffic.json records).
-ATTN_SOURCES = ("attn_cc.cu", "attn_mma.cu", "attn_tc.cu", "kvshot_api.cu", "kvshot_attn_common.cuh",
+ATTN_SOURCES = ("attn_cc.cu", "attn_f8.cu", "attn_mma.cu", "attn_tc.cu", "kvshot_api.cu", "kvshot_attn_common.cuh",
                 "kvshot_internal.h", "kvshot_tcgen05.cuh", "merge_append.cu")
 
 

@@ -15,7 +15,9 @@ namespace kvshot {
 
 // Defined in the kernel translation units.
 cudaError_t attn_cc_occupancy(int C, int* ctas_per_sm);
-cudaError_t attn_mma_occupancy(int m_tiles, int C, bool fp8, int* ctas_per_sm);
+cudaError_t attn_mma_occupancy(int m_tiles, int C, int* ctas_per_sm);
+cudaError_t attn_f8_occupancy(int rows_per_unit, int C, int* ctas_per_sm);
+int attn_f8_rows(int rows);  // rows per unit of the fp8 mma.sync kernel for a stack of `rows`
 cudaError_t attn_tc_occupancy(int C, int* ctas_per_sm);
 
 namespace {
@@ -54,7 +56,7 @@ bool encode_rows(CUtensorMap* map, const void* base, uint64_t rows, uint32_t box
 }
 
 // fp8 E4M3 target cache: one byte per element, whole 128-byte rows per box, under the 128-byte
-// swizzle (the m16n8k16 kernel decodes the codes from shared memory straight into MMA fragments).
+// swizzle.
 bool encode_rows_fp8(CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows) {
   auto fn = encode_fn();
   if (fn == nullptr) return false;
@@ -101,7 +103,7 @@ bool encode_rows_group3(CUtensorMap* map, const void* base, uint64_t rows) {
 
 constexpr int kMaxScaleExp = 64;
 
-enum class Kernel { kCudaCore, kMma, kTensorMemory };
+enum class Kernel { kCudaCore, kMma, kMmaF8, kTensorMemory };
 
 // Fixed cost, in 64-key tile times of one CTA, of splitting units across CTAs (piece epilogues
 // that stall the pipeline mid-stream, the merge kernel after the last CTA); measured on GB300.
@@ -114,6 +116,9 @@ constexpr int64_t kSplitCostTiles = 15;
 // 10.5 us on 8 CTAs; 2, 4, 6 or 8 tiles per CTA measured slower).  Large problems have hundreds of
 // tiles per CTA.
 constexpr int64_t kMinTilesPerCta = 3;
+// The fp8 mma.sync kernel's prefix tiles hold 128 keys (tiny chain, 8 units of 2 tiles: 16.5 us per call
+// with 3 tiles per CTA, 11.0 with 2, 12.1 with 1; KV-only chain, 17 tiles per unit: 16.7, 16.1, 16.3).
+constexpr int64_t kMinTilesPerCtaF8 = 2;
 
 }  // namespace
 
@@ -150,8 +155,7 @@ bool encode_q(CUtensorMap* map, const void* q, int C, int Nq, int hq, QBox qb) {
 
 struct Plan {
   Kernel kernel;
-  bool mma;
-  int m_tiles;        // mma path
+  int m_tiles;        // bf16 mma path
   int nq_box;         // tensor-memory path: draft nodes per 128-row block
   bool spread;        // tensor-memory path: 16 rows per TMEM lane quarter
   bool pair;          // tensor-memory path: two 128-row blocks per unit (stacks of more than 128 rows)
@@ -161,6 +165,7 @@ struct Plan {
   int num_ctas;
   int len_bound;
   int draft_tiles;
+  int prefix_tile;    // keys per prefix tile
   size_t off_lse, off_o, bytes;
 };
 
@@ -240,16 +245,17 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   //    per multi-layer-tree call at 16 rows (spread rows), 1.9x at 48 rows,
   //    3-4x for whole-tree stacks of 128-256 rows.
   const bool tc_ok = G <= 128 && 128 % G == 0;
-  // fp8 tiles: both kernels decode them (the tensor-memory kernel for stacks of up to 128 rows).  The
-  // producer warps' decode into shared memory for the tcgen05 MMAs is the faster path for 17-128 rows
-  // (hybrid tree per depth, 32-48 rows: 85 us against 103 us per call for the m16n8k16 kernel, which
-  // decodes in registers); at 16 rows and below the m16n8k16 kernel is far ahead (264 us against 476 us).
+  // fp8 tiles: the tcgen05 kernel decodes them into f16 tiles in shared memory (stacks of up to 128
+  // rows), attn_f8.cu into MMA fragments in registers.  Up to 16 rows the latter streams the codes at
+  // 0.84-0.89 of the copy peak (4 rows: 105 us per ragged-chain call, 16 rows: 179 us per multi-layer
+  // call, tcgen05 302 and 368 us); its MMAs pad and repeat with the rows, so from 17 rows the tcgen05
+  // kernel is ahead (hybrid tree, 32 and 48 rows: 65 and 66 us per call against 72 and 108 us).
   const bool fp8 = d->flags & KVSHOT_TARGET_FP8;
   const bool tc_auto = fp8 ? (rows > 16 && rows <= 128) : rows >= 16;
-  const Kernel automatic = (tc_auto && tc_ok) ? Kernel::kTensorMemory : Kernel::kMma;
+  const Kernel mma = fp8 ? Kernel::kMmaF8 : Kernel::kMma;
+  const Kernel automatic = (tc_auto && tc_ok) ? Kernel::kTensorMemory : mma;
   pl->kernel = force_cc ? Kernel::kCudaCore : force_tc ? Kernel::kTensorMemory
-                                           : force_mma ? Kernel::kMma : automatic;
-  pl->mma = pl->kernel == Kernel::kMma;
+                                           : force_mma ? mma : automatic;
   pl->m_tiles = 0;
   pl->nq_box = 0;
   pl->spread = false;
@@ -257,6 +263,8 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   if (pl->kernel == Kernel::kMma) {
     pl->m_tiles = std::min(kMmaMaxTiles, std::max(1, (rows + 15) / 16));
     pl->rows_per_unit = 16 * pl->m_tiles;
+  } else if (pl->kernel == Kernel::kMmaF8) {
+    pl->rows_per_unit = attn_f8_rows(rows);
   } else if (pl->kernel == Kernel::kTensorMemory) {
     pl->nq_box = std::max(1, std::min(d->n_query, 128 / G));
     pl->rows_per_unit = G * pl->nq_box;
@@ -272,16 +280,18 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   const int64_t cap = paged ? static_cast<int64_t>(d->max_pages_per_seq) * d->page_size : d->l_cap;
   pl->len_bound = static_cast<int>(std::min<int64_t>(d->max_seq_len, cap));
   pl->draft_tiles = (d->n_nodes + kTileKeys - 1) / kTileKeys;
+  pl->prefix_tile = pl->kernel == Kernel::kMmaF8 ? kF8PrefixTile : kTileKeys;
   // Upper bound on the tiles of any call with this descriptor (independent of the layout, so the
   // workspace size query and the call agree).
   const int64_t max_tiles =
-      units * ((static_cast<int64_t>(d->max_seq_len) + kTileKeys - 1) / kTileKeys + pl->draft_tiles);
+      units * ((static_cast<int64_t>(d->max_seq_len) + pl->prefix_tile - 1) / pl->prefix_tile + pl->draft_tiles);
   if (units >= INT_MAX / 2 || max_tiles >= INT_MAX / 2) return KVSHOT_ERR_UNSUPPORTED;
   pl->units = static_cast<int>(units);
   int grid = d->num_ctas;
   if (grid == 0) {
     int per_sm = 0;
-    const cudaError_t e = pl->kernel == Kernel::kMma ? attn_mma_occupancy(pl->m_tiles, d->num_caches, fp8, &per_sm)
+    const cudaError_t e = pl->kernel == Kernel::kMma ? attn_mma_occupancy(pl->m_tiles, d->num_caches, &per_sm)
+                          : pl->kernel == Kernel::kMmaF8 ? attn_f8_occupancy(pl->rows_per_unit, d->num_caches, &per_sm)
                           : pl->kernel == Kernel::kTensorMemory ? attn_tc_occupancy(d->num_caches, &per_sm)
                                                                  : attn_cc_occupancy(d->num_caches, &per_sm);
     const int sms = sm_count();
@@ -297,8 +307,10 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
       if (unit_tiles * (grid - units) < kSplitCostTiles * static_cast<int64_t>(grid)) grid = static_cast<int>(units);
     }
   }
-  if (d->num_ctas == 0)
-    grid = static_cast<int>(std::min<int64_t>(grid, (max_tiles + kMinTilesPerCta - 1) / kMinTilesPerCta));
+  if (d->num_ctas == 0) {
+    const int64_t least = pl->kernel == Kernel::kMmaF8 ? kMinTilesPerCtaF8 : kMinTilesPerCta;
+    grid = static_cast<int>(std::min<int64_t>(grid, (max_tiles + least - 1) / least));
+  }
   grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(grid, std::max<int64_t>(1, max_tiles))));
   pl->num_ctas = grid;
   const size_t slots = static_cast<size_t>(pl->units) + grid;
@@ -428,6 +440,7 @@ extern "C" kvshot_status kvshot_draft_attn(const kvshot_attn_desc* d, const void
   p.n_max = d->n_max;
   p.tree = tree ? 1 : 0;
   p.draft_tiles = pl.draft_tiles;
+  p.prefix_tile = pl.prefix_tile;
   const double scale = d->scale != 0.f ? static_cast<double>(d->scale) : 1.0 / std::sqrt(static_cast<double>(kHeadDim));
   p.qscale = static_cast<float>(scale * 1.4426950408889634);
   p.num_ctas = pl.num_ctas;
@@ -440,6 +453,7 @@ extern "C" kvshot_status kvshot_draft_attn(const kvshot_attn_desc* d, const void
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool pdl = (d->flags & KVSHOT_OVERLAP_PREVIOUS) != 0;
   cudaError_t e = pl.kernel == Kernel::kMma            ? launch_attn_mma(p, maps, pl.m_tiles, pdl, s)
+                  : pl.kernel == Kernel::kMmaF8        ? launch_attn_f8(p, maps, pdl, s)
                   : pl.kernel == Kernel::kTensorMemory ? launch_attn_tc(p, maps, pl.nq_box, pl.spread, pl.pair, pdl, s)
                                                        : launch_attn_cc(p, maps, pdl, s);
   if (e != cudaSuccess) return KVSHOT_ERR_CUDA;

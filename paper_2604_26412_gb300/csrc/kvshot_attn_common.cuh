@@ -271,13 +271,15 @@ __device__ __forceinline__ int clamp_len_of(const AttnParams& p, int L) {
 
 // s_len[c] = clamped L_c; s_base[c] = first global tile of cache c (prefix sum of
 // units x tiles per unit).  Whole block participates.  `len0` may hold
-// seq_lens[threadIdx.x], loaded early by the caller (-1: not loaded).
+// seq_lens[threadIdx.x], loaded early by the caller (-1: not loaded).  PK, here and below: keys
+// per prefix tile (draft tiles always hold kTileKeys).
+template <int PK = kTileKeys>
 __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int* s_base, int len0 = -1) {
   const int HR = p.hkv * p.row_blocks;
   for (int c = threadIdx.x; c < p.C; c += blockDim.x) {
     const int L = (c == static_cast<int>(threadIdx.x) && len0 >= 0) ? clamp_len_of(p, len0) : clamp_len(p, c);
     s_len[c] = L;
-    s_base[c + 1] = ((L + kTileKeys - 1) / kTileKeys + p.draft_tiles) * HR;
+    s_base[c + 1] = ((L + PK - 1) / PK + p.draft_tiles) * HR;
   }
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -308,12 +310,14 @@ struct Cursor {
   int L, pt, ut;          // prefix length, prefix tiles, tiles per unit
 };
 
+template <int PK = kTileKeys>
 __device__ __forceinline__ void cursor_load_cache(Cursor& cu, const AttnParams& p, const int* s_len) {
   cu.L = s_len[cu.c];
-  cu.pt = (cu.L + kTileKeys - 1) / kTileKeys;
+  cu.pt = (cu.L + PK - 1) / PK;
   cu.ut = cu.pt + p.draft_tiles;
 }
 
+template <int PK = kTileKeys>
 __device__ __forceinline__ Cursor cursor_begin(const AttnParams& p, const int* s_len, const int* s_base) {
   Cursor cu;
   const int total = s_base[p.C];
@@ -332,13 +336,14 @@ __device__ __forceinline__ Cursor cursor_begin(const AttnParams& p, const int* s
     else hi = mid - 1;
   }
   cu.c = lo;
-  cursor_load_cache(cu, p, s_len);
+  cursor_load_cache<PK>(cu, p, s_len);
   const int rem = cu.t - s_base[lo];
   cu.hr = rem / cu.ut;
   cu.lt = rem - cu.hr * cu.ut;
   return cu;
 }
 
+template <int PK = kTileKeys>
 __device__ __forceinline__ void cursor_next(Cursor& cu, const AttnParams& p, const int* s_len) {
   ++cu.t;
   if (++cu.lt == cu.ut) {
@@ -346,7 +351,7 @@ __device__ __forceinline__ void cursor_next(Cursor& cu, const AttnParams& p, con
     if (++cu.hr == p.hkv * p.row_blocks) {
       cu.hr = 0;
       ++cu.c;
-      if (cu.t < cu.t_end) cursor_load_cache(cu, p, s_len);
+      if (cu.t < cu.t_end) cursor_load_cache<PK>(cu, p, s_len);
     }
   }
 }
@@ -354,16 +359,17 @@ __device__ __forceinline__ void cursor_next(Cursor& cu, const AttnParams& p, con
 struct TileInfo {
   bool draft;   // draft tile (else prefix tile)
   int key0;     // first key: prefix token index, or draft slot
-  int nkeys;    // valid keys in the tile (1..TK)
+  int nkeys;    // valid keys in the tile
   bool first;   // first tile of this CTA's piece of the unit
   bool last;    // last tile of this CTA's piece of the unit
 };
 
+template <int PK = kTileKeys>
 __device__ __forceinline__ TileInfo tile_info(const Cursor& cu, const AttnParams& p) {
   TileInfo ti;
   ti.draft = cu.lt >= cu.pt;
-  ti.key0 = (ti.draft ? cu.lt - cu.pt : cu.lt) * kTileKeys;
-  ti.nkeys = min(kTileKeys, (ti.draft ? p.N : cu.L) - ti.key0);
+  ti.key0 = ti.draft ? (cu.lt - cu.pt) * kTileKeys : cu.lt * PK;
+  ti.nkeys = min(ti.draft ? kTileKeys : PK, (ti.draft ? p.N : cu.L) - ti.key0);
   ti.first = (cu.t == cu.t_begin) || cu.lt == 0;
   ti.last = (cu.t == cu.t_end - 1) || cu.lt == cu.ut - 1;
   return ti;
@@ -586,27 +592,23 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
                            full_bar, policy);
         }
       } else if (p.paged) {
-        // bf16: boxes of 64 dims per half; fp8 (p.fp8): one box of whole 128-byte rows, into the
-        // upper half of the tile (the lanes of half 1 skip), decoded from there by the consumers.
         const int br = p.box_rows;
         const int nbox = (nkeys + br - 1) / br;
-        if (lane == 0) mbar_arrive_expect_tx(full_bar, nbox * br * 128 * (p.fp8 ? 2 : 4));
-        if (i < nbox && !(p.fp8 && hf)) {
+        if (lane == 0) mbar_arrive_expect_tx(full_bar, nbox * br * 128 * 4);
+        if (i < nbox) {
           int pid = pids[0];
 #pragma unroll
           for (int k = 1; k < kTileKeys / 8; ++k)
             if (i == k) pid = pids[k];
           const int krow = key0 + i * br;
           const int y = (pid * p.hkv + h) * p.page_size + (krow % p.page_size);
-          const uint32_t d0 = p.fp8 ? kdst + kv * kKVTileBytes + kHalfBytes : dst;
-          tma_load_2d(d0 + i * br * 128, kv ? &maps.tv : &maps.tk, p.fp8 ? 0 : hf * 64, y, full_bar, policy);
+          tma_load_2d(dst + i * br * 128, kv ? &maps.tv : &maps.tk, hf * 64, y, full_bar, policy);
         }
       } else {
-        if (lane == 0) mbar_arrive_expect_tx(full_bar, kTileKeys * 128 * (p.fp8 ? 2 : 4));
-        if (i == 0 && !(p.fp8 && hf)) {
+        if (lane == 0) mbar_arrive_expect_tx(full_bar, kTileKeys * 128 * 4);
+        if (i == 0) {
           const int y = (cu.c * p.hkv + h) * p.l_cap + key0;
-          const uint32_t d0 = p.fp8 ? kdst + kv * kKVTileBytes + kHalfBytes : dst;
-          tma_load_2d(d0, kv ? &maps.tv : &maps.tk, p.fp8 ? 0 : hf * 64, y, full_bar, policy);
+          tma_load_2d(dst, kv ? &maps.tv : &maps.tk, hf * 64, y, full_bar, policy);
         }
       }
     }

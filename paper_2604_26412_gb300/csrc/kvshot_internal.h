@@ -27,6 +27,7 @@ constexpr int kTileKeys = 64;                         // TK
 constexpr int kHalfBytes = kTileKeys * 128;           // 64 dims x TK keys, bf16: one TMA-swizzled half
 constexpr int kKVTileBytes = 2 * kHalfBytes;          // one K (or V) tile
 constexpr int kStageBytes = 2 * kKVTileBytes;         // K + V
+constexpr int kF8PrefixTile = 128;                    // keys per prefix tile of the fp8 mma.sync kernel
 constexpr int kMaxCaches = 1024;
 constexpr int kMaxTreeNodes = 64;
 constexpr int kDraftBoxRows = 8;                      // draft K/V are loaded 8 rows per TMA box
@@ -74,9 +75,10 @@ struct AttnParams {
   int len_bound;            // min(max_seq_len, capacity): seq_lens are clamped to [0, len_bound]
   int N, Nq, n_max, tree;
   int draft_tiles;          // ceil(N / TK)
+  int prefix_tile;          // keys per prefix tile: TK, or kF8PrefixTile (fp8 mma.sync kernel)
   float qscale;             // softmax scale * log2(e): scores are kept in the log2 domain
   int num_ctas;             // persistent grid size
-  int fp8;                  // target K/V are e4m3 codes (KVSHOT_TARGET_FP8; m16n8k16 kernel only)
+  int fp8;                  // target K/V are e4m3 codes (KVSHOT_TARGET_FP8)
   int prefix_grouped;       // prefix tiles are staged in the grouped layout (tensor-memory kernel: draft tiles always;
                             // m16n8k16 kernel: draft tiles too)
   uint32_t wait_ns;         // limit on any one pipeline wait (desc->wait_limit_ns, default 2 s)
@@ -118,6 +120,7 @@ bool encode_bf16_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t 
 // launch with programmatic stream serialization (KVSHOT_OVERLAP_PREVIOUS).
 cudaError_t launch_attn_cc(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream);
 cudaError_t launch_attn_mma(const AttnParams& p, const TensorMaps& maps, int m_tiles, bool pdl, cudaStream_t stream);
+cudaError_t launch_attn_f8(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream);
 cudaError_t launch_attn_tc(const AttnParams& p, const TensorMaps& maps, int nq_box, bool spread, bool pair, bool pdl,
                            cudaStream_t stream);
 

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kMergeThreads, 6) merge_kernel(const __grid_co
   int cbase = 0, total = 0, ut = 0;
   for (int c0 = 0; c0 < p.C; c0 += 32) {
     const int cc = c0 + lane;
-    const int utc = cc < p.C ? (clamp_len(p, cc) + kTileKeys - 1) / kTileKeys + p.draft_tiles : 0;
+    const int utc = cc < p.C ? (clamp_len(p, cc) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles : 0;
     int below = cc < c ? utc * HR : 0, all = utc * HR;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

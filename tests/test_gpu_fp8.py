@@ -90,6 +90,20 @@ def test_fp8_tcgen05_matches_oracle_at_48_and_128_rows(nq):
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 tcgen05 nq={nq} ctas={num_ctas}")
 
 
+# The m16n8k16 kernel's row paddings (8, 16, 32, 48, 64 and a second 64-row block) at prefix lengths around its
+# 128-key tiles and 32-key chunks, and pages that tile 128 keys in every way (192: a tile spans two pages).
+@pytest.mark.parametrize("nq,hq,hkv", [(1, 32, 8), (2, 32, 8), (3, 15, 5), (5, 32, 8), (8, 32, 8), (11, 32, 8),
+                                       (15, 32, 8), (17, 32, 8)])
+@pytest.mark.parametrize("paged,page", [(False, 16), (True, 8), (True, 192), (True, 256)])
+def test_fp8_m16n8k16_rows_tiles_and_pages(nq, hq, hkv, paged, page):
+    case = ((127, 128, 129, 31, 33, 0, 385), (17,), True, paged, page, hq, hkv, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=100 + nq + page)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for num_ctas in (0, 5):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, kvshot.KVSHOT_FORCE_MMA, num_ctas)
+        gh.compare(out, lse, ref_out, ref_lse, f"fp8 mma nq={nq} {hq}/{hkv} page={page if paged else 0} ctas={num_ctas}")
+
+
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
     spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(((2000, 900), (4, 4), True, True, 16, 32, 8, 4), seed=21)
     a = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
