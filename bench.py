@@ -385,7 +385,7 @@ def call_roofline(step, inp, spec: wl.Spec, stream, ms_per_step: float, hbm_peak
         kernels = ["m16n8k16"]
     else:  # the library's automatic choice (kvshot_api.cu make_plan)
         def auto(rows):
-            tc = (16 < rows <= 128) if target_elem == 1 else rows >= 16
+            tc = rows > 16 if target_elem == 1 else rows >= 16
             return "tcgen05" if tc and 128 % G == 0 else "m16n8k16"
         kernels = sorted({auto(G * lv) for lv in levels})
     traffic = None

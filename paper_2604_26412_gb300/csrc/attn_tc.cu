@@ -32,7 +32,7 @@
 // 16-token pages takes 4 boxes per tensor instead of 8.  Ring depths (5 K,
 // 6 V) were measured on GB300: the bytes in flight per SM that the rings
 // allow bound how fast one CTA streams.
-// fp8 target cache (dense and spread rows; the default for 17..128 rows): the
+// fp8 target cache (dense and spread rows; the default from 17 rows, in blocks of up to 128): the
 // producer warps land the e4m3 codes of each tile in a landing slot, and the
 // softmax warpgroup between tiles decodes them into the f16 K and V ring tiles
 // (three tiles ahead of the tile it takes next); q and the draft tiles are

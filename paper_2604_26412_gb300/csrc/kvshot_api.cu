@@ -229,7 +229,8 @@ kvshot_status check_attn_desc(const kvshot_attn_desc* d, bool paged) {
   return KVSHOT_OK;
 }
 
-kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
+// `small_blocks`: an fp8 stack of more than 128 rows takes attn_f8.cu's 64-row blocks.
+kvshot_status make_plan_for(const kvshot_attn_desc* d, bool paged, bool small_blocks, Plan* pl) {
   const int G = d->hq / d->hkv;
   const int rows = G * d->n_query;
   const bool force_cc = d->flags & KVSHOT_FORCE_CC, force_tc = d->flags & KVSHOT_FORCE_TC;
@@ -245,13 +246,16 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   //    per multi-layer-tree call at 16 rows (spread rows), 1.9x at 48 rows,
   //    3-4x for whole-tree stacks of 128-256 rows.
   const bool tc_ok = G <= 128 && 128 % G == 0;
-  // fp8 tiles: the tcgen05 kernel decodes them into f16 tiles in shared memory (stacks of up to 128
-  // rows), attn_f8.cu into MMA fragments in registers.  Up to 16 rows the latter streams the codes at
+  // fp8 tiles: the tcgen05 kernel decodes them into f16 tiles in shared memory,
+  // attn_f8.cu into MMA fragments in registers.  Up to 16 rows the latter streams the codes at
   // 0.84-0.89 of the copy peak (4 rows: 105 us per ragged-chain call, 16 rows: 179 us per multi-layer
   // call, tcgen05 302 and 368 us); its MMAs pad and repeat with the rows, so from 17 rows the tcgen05
-  // kernel is ahead (hybrid tree, 32 and 48 rows: 65 and 66 us per call against 72 and 108 us).
+  // kernel is ahead (hybrid tree, 32 and 48 rows: 65 and 66 us per call against 72 and 108 us).  Stacks
+  // of more than 128 rows take it in 128-row blocks (the paired kernel has no fp8 form): reading the
+  // codes once per block still beats the 64-row blocks of attn_f8.cu (whole hybrid tree, 256 rows:
+  // 179 us against 350 us; with the 64-row blocks of the bf16 kernel's fp8 form it was 529 us).
   const bool fp8 = d->flags & KVSHOT_TARGET_FP8;
-  const bool tc_auto = fp8 ? (rows > 16 && rows <= 128) : rows >= 16;
+  const bool tc_auto = fp8 ? rows > 16 && !(small_blocks && rows > 128) : rows >= 16;
   const Kernel mma = fp8 ? Kernel::kMmaF8 : Kernel::kMma;
   const Kernel automatic = (tc_auto && tc_ok) ? Kernel::kTensorMemory : mma;
   pl->kernel = force_cc ? Kernel::kCudaCore : force_tc ? Kernel::kTensorMemory
@@ -266,11 +270,16 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   } else if (pl->kernel == Kernel::kMmaF8) {
     pl->rows_per_unit = attn_f8_rows(rows);
   } else if (pl->kernel == Kernel::kTensorMemory) {
-    pl->nq_box = std::max(1, std::min(d->n_query, 128 / G));
+    const int most = 128 / G;  // draft nodes in a block of up to 128 rows
+    pl->nq_box = std::max(1, std::min(d->n_query, most));
+    if (fp8 && d->n_query > most) {  // blocks of equal size
+      const int blocks = (d->n_query + most - 1) / most;
+      pl->nq_box = (d->n_query + blocks - 1) / blocks;
+    }
     pl->rows_per_unit = G * pl->nq_box;
     pl->spread = pl->rows_per_unit <= kSpreadMaxRows;
-    // More than 128 rows: each unit takes two 128-row blocks, so every K/V tile feeds both.
-    pl->pair = rows > 128;
+    // More than 128 rows: each unit takes two 128-row blocks, so every K/V tile feeds both (bf16 cache).
+    pl->pair = rows > 128 && !fp8;
     if (pl->pair) pl->rows_per_unit = 2 * 128;
   } else {
     pl->rows_per_unit = kCcRows;
@@ -317,6 +326,15 @@ kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
   pl->off_lse = 0;
   pl->off_o = pl->off_lse + round_up(sizeof(float) * slots * pl->rows_per_unit, 256);
   pl->bytes = pl->off_o + sizeof(float) * slots * pl->rows_per_unit * kHeadDim;
+  return KVSHOT_OK;
+}
+
+kvshot_status make_plan(const kvshot_attn_desc* d, bool paged, Plan* pl) {
+  if (kvshot_status st = make_plan_for(d, paged, false, pl)) return st;
+  // fp8 stacks of more than 128 rows: 128-row blocks need up to 5 MB more scratch than 64-row blocks, which
+  // keep the largest of them inside the scratch of kvshot_draft_attn_static.
+  if ((d->flags & KVSHOT_TARGET_FP8) && d->hq / d->hkv * d->n_query > 128 && pl->bytes > KVSHOT_STATIC_WORKSPACE_BYTES)
+    return make_plan_for(d, paged, true, pl);
   return KVSHOT_OK;
 }
 

@@ -29,7 +29,7 @@ CASES = [
     ((333, 5), (3, 3), True, False, 16, 8, 8, 3),                 # G = 1
     ((65,), tuple([1] * 70), False, False, 16, 4, 4, 2),          # chain with N = 70 > one draft tile
     ((203, 64), tuple([1] * 40), False, False, 16, 32, 8, 32),    # 128 dense rows, contiguous l_cap % 8 != 0
-    ((300, 200), (8, 12, 12, 12), True, True, 16, 32, 8, 40),     # 160 rows: m16n8k16 only (no paired fp8 blocks)
+    ((300, 200), (8, 12, 12, 12), True, True, 16, 32, 8, 40),     # 160 rows: two blocks
 ]
 
 
@@ -102,6 +102,18 @@ def test_fp8_m16n8k16_rows_tiles_and_pages(nq, hq, hkv, paged, page):
     for num_ctas in (0, 5):
         out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, kvshot.KVSHOT_FORCE_MMA, num_ctas)
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 mma nq={nq} {hq}/{hkv} page={page if paged else 0} ctas={num_ctas}")
+
+
+# More than 128 rows: blocks of up to 128 rows on the tcgen05 kernel (2 x 80, 2 x 128, 2 x 68 rows
+# with an idle node, 3 x 88, 2 x 96 rows of G = 32).
+@pytest.mark.parametrize("nq,hq,hkv", [(40, 32, 8), (64, 32, 8), (33, 32, 8), (33, 64, 8), (6, 64, 2)])
+def test_fp8_stacks_of_more_than_128_rows(nq, hq, hkv):
+    case = ((700, 65, 0), (8, 12, 12, 12, 12, 8), True, True, 16, hq, hkv, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=200 + nq)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for num_ctas in (0, 5):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0, num_ctas)
+        gh.compare(out, lse, ref_out, ref_lse, f"fp8 blocks nq={nq} {hq}/{hkv} ctas={num_ctas}")
 
 
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
