@@ -5,6 +5,8 @@
 //   * append: RoPE on the drafter's new q and k, then the store of k / v into
 //             the draft slots (App. B: draft positions j > t take the drafter's
 //             own K/V; Sec. 3.2: RoPE re-applied to drafted keys).
+#include <algorithm>
+
 #include "kvshot_attn_common.cuh"
 
 namespace kvshot {
@@ -31,6 +33,10 @@ __global__ void __launch_bounds__(kMergeThreads, 6) merge_kernel(const __grid_co
   const int u = blockIdx.x / blocks_per_unit;
   const int r = (blockIdx.x - u * blocks_per_unit) * kMergeRows + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  // Rows of unsplit units leave without waiting for the attention grid, so CTA 0 waits for it in any case:
+  // a kernel that depends on this grid alone (the next append) then comes after the attention too.
+  if (blockIdx.x == 0) wait_for_prerequisite_grid();
+  if (threadIdx.x == 0) allow_dependent_launch();
   const int HR = p.hkv * p.row_blocks;
   const int c = u / HR, hr = u - c * HR;
   const int h = hr / p.row_blocks, rb = hr - h * p.row_blocks;
@@ -107,90 +113,243 @@ __global__ void __launch_bounds__(kMergeThreads, 6) merge_kernel(const __grid_co
   if (lane == 0) p.lse[orow] = Lsum > 0.f ? (M + log2f(Lsum)) * 0.69314718055994531f : -INFINITY;
 }
 
-constexpr int kAppendThreads = 256;
+constexpr int kAppendThreads = 128;
+// A node is shared out over up to kAppendSplits CTAs while the grid stays within kAppendCtas; from twice as many
+// nodes, a CTA takes kAppendGroup.  (Within 256 CTAs: 192 nodes 4.5 us, 1024 nodes 14.1 us; 512: 4.6 and 12.4 us;
+// 1024 nodes in CTAs of 4 13.7, of 1 10.8 us alone but 0.7 us slower with the attention behind them.)
+constexpr int kAppendCtas = 512;
+constexpr int kAppendSplits = 4;
+constexpr int kAppendGroup = 2;
 
-// One rotated component of RoPE, x' = a * cos - b * sin (sgn = -1) or
-// y' = b * cos + a * sin (sgn = +1), rounded to bf16 as the fp64 evaluation
-// rounds.  The fp32 value r differs from the exact a c + sgn b s by at most
-// 2^-24 (|a| + 2 |b| + |r|) (cos/sin rounded to fp32, one product and one fma
-// rounded); when r lies farther than twice that from every bf16 rounding
-// midpoint both round alike, otherwise the component is recomputed in fp64.
-__device__ __forceinline__ __nv_bfloat16 rope_bf16(float a, float b, float c32, float s32, double c, double s,
-                                                   float sgn) {
-  const float r = fmaf(a, c32, sgn * (b * s32));
-  const uint32_t u = __float_as_uint(r);
-  const int e = static_cast<int>((u >> 23) & 0xFFu);
-  const float bound = 0x1p-23f * (fabsf(a) + 2.f * fabsf(b) + fabsf(r));
-  if (e >= 40) {
-    const float ulp = __uint_as_float(static_cast<uint32_t>(e - 23) << 23);  // 2^(e - 150), fp32 spacing at r
-    const float dist = fabsf(static_cast<float>(static_cast<int>(u & 0xFFFFu) - 0x8000)) * ulp;
-    if (dist > bound) return __float2bfloat16_rn(r);
-  }
-  const double da = a, db = b;
-  return __double2bfloat16(sgn < 0.f ? da * c - db * s : da * c + db * s);
+__device__ __noinline__ void sincos_far(double theta, double* sn, double* cs) { sincos(theta, sn, cs); }
+
+// An unevaluated sum of two fp32 values, |l| <= half an ulp of h.
+struct Pair {
+  float h, l;
+};
+__host__ __device__ constexpr Pair pair_of(double x) {
+  return Pair{static_cast<float>(x), static_cast<float>(x - static_cast<double>(static_cast<float>(x)))};
+}
+// a + b for |a.h| >= |b.h| (or a of larger exponent), to ~2^-46 of the larger.
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float e = __fadd_rn(__fadd_rn(b.h, -__fadd_rn(s, -a.h)), __fadd_rn(a.l, b.l));
+  const float h = __fadd_rn(s, e);
+  return Pair{h, __fadd_rn(e, -__fadd_rn(h, -s))};
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return Pair{p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
 }
 
-// One CTA per (cache, new node).  Work item = (head, 16-byte chunk j0 of the
-// first half): it rotates dims j0..j0+7 together with their partners +64.
-__global__ void __launch_bounds__(kAppendThreads) append_kernel(const __grid_constant__ AppendParams a) {
-  // An attention call launched with KVSHOT_OVERLAP_PREVIOUS may start its prologue meanwhile.
+// sin and cos of theta as pairs, to 2^-40 absolute: Cody-Waite reduction to [-pi/4, pi/4] in fp64 by two fused
+// steps (pi/2 as an fp64 and its remainder; below 2^40 each step's only error is the rounding of its small
+// result), then the Taylor polynomials with their last coefficients in fp32 and the others in fp32 pairs.  An SM
+// executes two fp64 lanes per clock and 128 fp32 ones: the angles of a node take 9 fp64 operations per
+// frequency, where fp64 polynomials take 31 (4.9 of the 14.6 us of a 1024-node append) and the library more.
+__device__ __forceinline__ void sincos_pair(double theta, Pair* sn, Pair* cs) {
+  if (!(fabs(theta) < 0x1p40)) {
+    double s, c;
+    sincos_far(theta, &s, &c);
+    *sn = Pair{static_cast<float>(s), static_cast<float>(s - static_cast<double>(static_cast<float>(s)))};
+    *cs = Pair{static_cast<float>(c), static_cast<float>(c - static_cast<double>(static_cast<float>(c)))};
+    return;
+  }
+  const double n = rint(theta * 0.63661977236758134308);
+  double rd = fma(-n, 1.5707963267948965580, theta);
+  rd = fma(-n, 6.1232339957367658860e-17, rd);
+  const float rh = static_cast<float>(rd);
+  const Pair r{rh, static_cast<float>(rd - static_cast<double>(rh))};
+  const int q = static_cast<int>(static_cast<long long>(n) & 3);
+  const Pair z = pair_mul(r, r);
+  constexpr Pair s1 = pair_of(-1.0 / 6.0), s2 = pair_of(1.0 / 120.0), s3 = pair_of(-1.0 / 5040.0);
+  const float s4 = fmaf(z.h, fmaf(z.h, 1.6059044e-10f, -2.5052108e-8f), 2.7557319e-6f);  // 1/9!, -1/11!, 1/13!
+  Pair s = pair_add(s3, Pair{z.h * s4, 0.f});
+  s = pair_add(s2, pair_mul(z, s));
+  s = pair_add(s1, pair_mul(z, s));
+  s = pair_add(r, pair_mul(pair_mul(r, z), s));
+  constexpr Pair c1{-0.5f, 0.f}, c2 = pair_of(1.0 / 24.0), c3 = pair_of(-1.0 / 720.0), one{1.f, 0.f};
+  const float c4 = fmaf(z.h, fmaf(z.h, fmaf(z.h, -1.1470746e-11f, 2.0876757e-9f), -2.7557319e-7f), 2.4801587e-5f);
+  Pair c = pair_add(c3, Pair{z.h * c4, 0.f});
+  c = pair_add(c2, pair_mul(z, c));
+  c = pair_add(c1, pair_mul(z, c));
+  c = pair_add(one, pair_mul(z, c));
+  const Pair a = (q & 1) ? c : s, b = (q & 1) ? s : c;
+  *sn = (q & 2) ? Pair{-a.h, -a.l} : a;
+  *cs = (q == 1 || q == 2) ? Pair{-b.h, -b.l} : b;
+}
+
+// The append kernels are launched with programmatic stream serialization: their CTAs may be placed while the
+// preceding kernel still runs, and touch memory only once it has completed.  A following attention call
+// launched with KVSHOT_OVERLAP_PREVIOUS may start its prologue from here on: everything before this kernel
+// is complete by now.
+__device__ __forceinline__ void begin_after_previous() {
+  wait_for_prerequisite_grid();
   if (threadIdx.x == 0) allow_dependent_launch();
-  __shared__ double s_cos[kHeadDim / 2], s_sin[kHeadDim / 2];
-  const int c = blockIdx.x / a.n_new, i = blockIdx.x - (blockIdx.x / a.n_new) * a.n_new;
-  const int pos = a.positions[static_cast<size_t>(c) * a.n_new + i];
-  for (int j = threadIdx.x; j < kHeadDim / 2; j += blockDim.x) {
-    double sn, cs;
-    sincos(static_cast<double>(pos) * a.inv_freq[j], &sn, &cs);
-    s_cos[j] = cs;
-    s_sin[j] = sn;
+}
+
+// cos (or sin) of an angle as two fp32 values: the first with 16 significant bits, so that its product with a
+// bf16 is exact, and the rest.
+__device__ __forceinline__ float2 split16(Pair x) {
+  const float hi = __uint_as_float(__float_as_uint(x.h) & 0xffffff00u);
+  return make_float2(hi, __fadd_rn(__fadd_rn(x.h, -hi), x.l));
+}
+// Place of frequency j in a table of float4: eight lanes that read entries 8 apart hit all banks once.
+__device__ __forceinline__ constexpr int angle_at(int j) { return j + (j >> 3); }
+
+// The bits of the bf16 nearest to a * cos + sgn * b * sin, evaluated in fp64 and rounded once.
+__device__ __noinline__ uint32_t rope_bf16_fp64(float a, float b, double theta, float sgn) {
+  double s, c;
+  sincos_far(theta, &s, &c);
+  return __bfloat16_as_ushort(__double2bfloat16(static_cast<double>(a) * c + sgn * (static_cast<double>(b) * s)));
+}
+
+// One rotated component of RoPE, x' = a * cos + sgn * b * sin: the exact value is r + res to 2^-37 (|a| + |b|).
+// a, b are bf16, so a c.x and b s.x are exact in fp32; u + e is their exact sum (two-sum).
+struct Rotated {
+  float r, res;
+};
+__device__ __forceinline__ Rotated rotate(float a, float b, float2 c, float2 s, float sgn) {
+  const float p = a * c.x, q = sgn * (b * s.x);
+  const float u = __fadd_rn(p, q);
+  const float bb = __fadd_rn(u, -p);
+  const float e = __fadd_rn(__fadd_rn(p, -__fadd_rn(u, -bb)), __fadd_rn(q, -bb));
+  const float v = __fadd_rn(e, fmaf(a, c.y, sgn * (b * s.y)));
+  const float r = __fadd_rn(u, v);
+  return Rotated{r, __fadd_rn(v, -__fadd_rn(r, -u))};
+}
+
+// With |r| >= 2^-13 (|a| + |b|) that error is under one fp32 ulp of r, so unless r's low 16 bits are within
+// two of the rounding midpoint 0x8000, r rounds to the same bf16 as the exact value: (bits(r) + 0x8000) >> 16.
+__device__ __forceinline__ bool rounds_alike(float r, float least) {
+  return ((__float_as_uint(r) + 0x8002u) & 0xffffu) > 4u && fabsf(r) >= least;
+}
+
+// The bf16 of a component that does not (one in 5,000).  d is its distance past the midpoint above the truncated
+// bf16, so |d| beyond the error decides the rounding.  Only the rest (one in millions), values so small that the
+// products are not exact, infinities and NaN are evaluated in fp64.
+__device__ __noinline__ uint32_t rope_bf16_near(float a, float b, float4 cs, float sgn, double theta) {
+  const float2 c = make_float2(cs.x, cs.y), s = make_float2(cs.z, cs.w);
+  const Rotated x = rotate(a, b, c, s, sgn);
+  const float m = fabsf(a) + fabsf(b);
+  if (m == 0.f) return __float_as_uint(__fadd_rn(a * c.x, sgn * (b * s.x))) >> 16;  // a zero, signed as in fp64
+  const uint32_t w = __float_as_uint(x.r), e = (w >> 23) & 0xffu;
+  if (e > 60u && e < 255u) {
+    const float ulp = __uint_as_float((e - 23u) << 23);  // fp32 spacing at r
+    const float d = fmaf(static_cast<float>(static_cast<int>(w & 0xffffu) - 0x8000), ulp, x.r < 0.f ? -x.res : x.res);
+    if (fabsf(d) > 0x1p-37f * m) return (w >> 16) + (d > 0.f ? 1u : 0u);
   }
-  __syncthreads();
-  const int heads = a.hq + a.hkv;
-  for (int w = threadIdx.x; w < heads * 8; w += blockDim.x) {
-    const int head = w >> 3, j0 = (w & 7) * 8;
-    const __nv_bfloat16* src;
-    __nv_bfloat16* dst;
-    if (head < a.hq) {
-      const size_t off = ((static_cast<size_t>(c) * a.n_new + i) * a.hq + head) * kHeadDim;
-      src = a.q_in + off;
-      dst = a.q_out + off;
-    } else {
-      const int kh = head - a.hq;
-      src = a.k_in + ((static_cast<size_t>(c) * a.n_new + i) * a.hkv + kh) * kHeadDim;
-      dst = a.draft_k + ((static_cast<size_t>(c) * a.hkv + kh) * a.n_max + a.n0 + i) * kHeadDim;
-    }
-    const uint4 lo = *reinterpret_cast<const uint4*>(src + j0);
-    const uint4 hi = *reinterpret_cast<const uint4*>(src + 64 + j0);
-    const uint32_t wl[4] = {lo.x, lo.y, lo.z, lo.w}, wh[4] = {hi.x, hi.y, hi.z, hi.w};
-    uint32_t ol[4], oh[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      __nv_bfloat16 rl[2], rh[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int j = j0 + 2 * k + e;
-        const float x = e ? bf16_hi(wl[k]) : bf16_lo(wl[k]);
-        const float y = e ? bf16_hi(wh[k]) : bf16_lo(wh[k]);
-        const double cs = s_cos[j], sn = s_sin[j];
-        const float c32 = static_cast<float>(cs), s32 = static_cast<float>(sn);
-        rl[e] = rope_bf16(x, y, c32, s32, cs, sn, -1.f);
-        rh[e] = rope_bf16(y, x, c32, s32, cs, sn, 1.f);
-      }
-      ol[k] = static_cast<uint32_t>(__bfloat16_as_ushort(rl[0])) |
-              (static_cast<uint32_t>(__bfloat16_as_ushort(rl[1])) << 16);
-      oh[k] = static_cast<uint32_t>(__bfloat16_as_ushort(rh[0])) |
-              (static_cast<uint32_t>(__bfloat16_as_ushort(rh[1])) << 16);
-    }
-    *reinterpret_cast<uint4*>(dst + j0) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
-    *reinterpret_cast<uint4*>(dst + 64 + j0) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
-  }
-  // V: plain copy into the draft slot.
-  for (int w = threadIdx.x; w < a.hkv * 16; w += blockDim.x) {
+  return rope_bf16_fp64(a, b, theta, sgn);
+}
+
+// Grid (group of a.group consecutive nodes, split): a node's heads and V chunks are shared out over gridDim.y
+// CTAs when there are few nodes; a CTA takes several nodes when there are many, and forms the angles again only
+// where the position changes (the nodes of one tree level share theirs).
+struct AppendNode {
+  int c, i;
+  size_t row;  // (cache, node)
+};
+__device__ __forceinline__ AppendNode append_node(const AppendParams& a, int node) {
+  AppendNode t;
+  t.c = node / a.n_new;
+  t.i = node - t.c * a.n_new;
+  t.row = static_cast<size_t>(node);
+  return t;
+}
+__device__ __forceinline__ int share(int n, int k) {  // first of the k-th CTA's items of n
+  return static_cast<int>(static_cast<unsigned>(n) * static_cast<unsigned>(k) / gridDim.y);
+}
+// V: plain copy into the draft slot.
+__device__ __forceinline__ void append_v(const AppendParams& a, const AppendNode& t) {
+  const int w1 = share(a.hkv * 16, blockIdx.y + 1);
+  for (int w = share(a.hkv * 16, blockIdx.y) + threadIdx.x; w < w1; w += kAppendThreads) {
     const int kh = w >> 4, ch = w & 15;
-    const uint4 v = *reinterpret_cast<const uint4*>(
-        a.v_in + ((static_cast<size_t>(c) * a.n_new + i) * a.hkv + kh) * kHeadDim + ch * 8);
-    *reinterpret_cast<uint4*>(a.draft_v + ((static_cast<size_t>(c) * a.hkv + kh) * a.n_max + a.n0 + i) * kHeadDim +
+    const uint4 v = *reinterpret_cast<const uint4*>(a.v_in + (t.row * a.hkv + kh) * kHeadDim + ch * 8);
+    *reinterpret_cast<uint4*>(a.draft_v + ((static_cast<size_t>(t.c) * a.hkv + kh) * a.n_max + a.n0 + t.i) * kHeadDim +
                               ch * 8) = v;
+  }
+}
+
+// Work item = (head, 16-byte chunk j0 of the first half): it rotates dims j0..j0+7 together with their
+// partners +64.  Latency bound at a few nodes (a thread's first loads go out before the angles are formed, the
+// rotations of an item have no branch between them), and by the rotation's instructions at many.  Per call, back
+// to back in a graph: 1 node 2.4 us, 16 x 12 nodes 4.5 us, 16 x 64 nodes 12.4 us; with fp64 angles read per
+// component, converted there, and an error bound per component: 6.4, 7.1 and 20.8 us.
+__global__ void __launch_bounds__(kAppendThreads, 5) append_kernel(const __grid_constant__ AppendParams a) {
+  begin_after_previous();
+  __shared__ float4 angles[angle_at(kHeadDim / 2)];  // cos and sin, split16
+  const int items = (a.hq + a.hkv) * 8, w0 = share(items, blockIdx.y), w1 = share(items, blockIdx.y + 1);
+  const int node0 = blockIdx.x * a.group, node1 = min(a.C * a.n_new, node0 + a.group);
+  int had = -1;  // the position whose angles are in shared memory
+  for (int node = node0; node < node1; ++node) {
+    const AppendNode t = append_node(a, node);
+    const int pos = a.positions[t.row];
+    auto source = [&](int w) {
+      const int head = w >> 3;
+      return (head < a.hq ? a.q_in + (t.row * a.hq + head) * kHeadDim
+                          : a.k_in + (t.row * a.hkv + head - a.hq) * kHeadDim) + (w & 7) * 8;
+    };
+    uint4 lo = make_uint4(0, 0, 0, 0), hi = lo;
+    int w = w0 + threadIdx.x;
+    if (w < w1) {
+      const __nv_bfloat16* src = source(w);
+      lo = *reinterpret_cast<const uint4*>(src);
+      hi = *reinterpret_cast<const uint4*>(src + 64);
+    }
+    append_v(a, t);
+    if (node == node0 || pos != had) {  // the same for the whole CTA
+      if (node != node0) __syncthreads();
+      if (threadIdx.x < kHeadDim / 2) {
+        Pair sn, cs;
+        sincos_pair(static_cast<double>(pos) * a.inv_freq[threadIdx.x], &sn, &cs);
+        const float2 c = split16(cs), s = split16(sn);
+        angles[angle_at(threadIdx.x)] = make_float4(c.x, c.y, s.x, s.y);
+      }
+      __syncthreads();
+      had = pos;
+    }
+    while (w < w1) {
+      const int head = w >> 3, j0 = (w & 7) * 8;
+      __nv_bfloat16* dst =
+          head < a.hq ? a.q_out + (t.row * a.hq + head) * kHeadDim
+                      : a.draft_k + ((static_cast<size_t>(t.c) * a.hkv + head - a.hq) * a.n_max + a.n0 + t.i) * kHeadDim;
+      const uint32_t wl[4] = {lo.x, lo.y, lo.z, lo.w}, wh[4] = {hi.x, hi.y, hi.z, hi.w};
+      w += kAppendThreads;
+      if (w < w1) {  // the next item
+        const __nv_bfloat16* src = source(w);
+        lo = *reinterpret_cast<const uint4*>(src);
+        hi = *reinterpret_cast<const uint4*>(src + 64);
+      }
+      const float4* table = angles + angle_at(j0);  // j0 is a multiple of 8
+      // All sixteen components at once, without branches; the few that need a closer look are done again.
+      uint32_t ol[4], oh[4], near = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float x = k & 1 ? bf16_hi(wl[k >> 1]) : bf16_lo(wl[k >> 1]);
+        const float y = k & 1 ? bf16_hi(wh[k >> 1]) : bf16_lo(wh[k >> 1]);
+        const float4 cs = table[k];
+        const float2 c = make_float2(cs.x, cs.y), s = make_float2(cs.z, cs.w);
+        const float least = fmaxf((fabsf(x) + fabsf(y)) * 0x1p-13f, 0x1p-60f);
+        const float rl = rotate(x, y, c, s, -1.f).r, rh = rotate(y, x, c, s, 1.f).r;
+        near |= (rounds_alike(rl, least) ? 0u : 1u << k) | (rounds_alike(rh, least) ? 0u : 256u << k);
+        const uint32_t bl = __float_as_uint(rl) + 0x8000u, bh = __float_as_uint(rh) + 0x8000u;
+        ol[k >> 1] = k & 1 ? __byte_perm(ol[k >> 1], bl, 0x7632) : bl;
+        oh[k >> 1] = k & 1 ? __byte_perm(oh[k >> 1], bh, 0x7632) : bh;
+      }
+      if (near != 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float x = k & 1 ? bf16_hi(wl[k >> 1]) : bf16_lo(wl[k >> 1]);
+          const float y = k & 1 ? bf16_hi(wh[k >> 1]) : bf16_lo(wh[k >> 1]);
+          const uint32_t into = k & 1 ? 0x5410u : 0x3254u;  // the new half word over the high or the low one
+          const double theta = static_cast<double>(pos) * a.inv_freq[j0 + k];
+          if (near >> k & 1u) ol[k >> 1] = __byte_perm(ol[k >> 1], rope_bf16_near(x, y, table[k], -1.f, theta), into);
+          if (near >> (8 + k) & 1u) oh[k >> 1] = __byte_perm(oh[k >> 1], rope_bf16_near(y, x, table[k], 1.f, theta), into);
+        }
+      }
+      *reinterpret_cast<uint4*>(dst + j0) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
+      *reinterpret_cast<uint4*>(dst + 64 + j0) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+    }
   }
 }
 
@@ -198,59 +357,63 @@ __global__ void __launch_bounds__(kAppendThreads) append_kernel(const __grid_con
 // holding dims 2l, 2l + 1 and their RoPE partners + 64.  x <- x / sqrt(mean(x^2) + eps) * w (w the
 // head-dim weights), then the rotation; fp32 throughout, one rounding to bf16.
 __global__ void __launch_bounds__(kAppendThreads) append_qknorm_kernel(const __grid_constant__ AppendParams a) {
-  if (threadIdx.x == 0) allow_dependent_launch();
+  begin_after_previous();
   __shared__ float s_cos[kHeadDim / 2], s_sin[kHeadDim / 2];
-  const int c = blockIdx.x / a.n_new, i = blockIdx.x - (blockIdx.x / a.n_new) * a.n_new;
-  const int pos = a.positions[static_cast<size_t>(c) * a.n_new + i];
-  for (int j = threadIdx.x; j < kHeadDim / 2; j += blockDim.x) {
-    double sn, cs;
-    sincos(static_cast<double>(pos) * a.inv_freq[j], &sn, &cs);
-    s_cos[j] = static_cast<float>(cs);
-    s_sin[j] = static_cast<float>(sn);
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = 2 * lane;
-  for (int head = warp; head < a.hq + a.hkv; head += kAppendThreads / 32) {
-    const __nv_bfloat16* src;
-    __nv_bfloat16* dst;
-    const __nv_bfloat16* w;
-    if (head < a.hq) {
-      const size_t off = ((static_cast<size_t>(c) * a.n_new + i) * a.hq + head) * kHeadDim;
-      src = a.q_in + off;
-      dst = a.q_out + off;
-      w = a.q_norm_w;
-    } else {
-      const int kh = head - a.hq;
-      src = a.k_in + ((static_cast<size_t>(c) * a.n_new + i) * a.hkv + kh) * kHeadDim;
-      dst = a.draft_k + ((static_cast<size_t>(c) * a.hkv + kh) * a.n_max + a.n0 + i) * kHeadDim;
-      w = a.k_norm_w;
+  const int heads = a.hq + a.hkv, h0 = share(heads, blockIdx.y), h1 = share(heads, blockIdx.y + 1);
+  const int lane = threadIdx.x & 31, j = 2 * lane;
+  const int node0 = blockIdx.x * a.group, node1 = min(a.C * a.n_new, node0 + a.group);
+  int had = -1;
+  for (int node = node0; node < node1; ++node) {
+    const AppendNode t = append_node(a, node);
+    const int pos = a.positions[t.row];
+    auto source = [&](int hd) {
+      return (hd < a.hq ? a.q_in + (t.row * a.hq + hd) * kHeadDim : a.k_in + (t.row * a.hkv + hd - a.hq) * kHeadDim) + j;
+    };
+    int head = h0 + (threadIdx.x >> 5);
+    uint32_t lo = 0, hi = 0;
+    if (head < h1) {
+      lo = *reinterpret_cast<const uint32_t*>(source(head));
+      hi = *reinterpret_cast<const uint32_t*>(source(head) + 64);
     }
-    const uint32_t lo = *reinterpret_cast<const uint32_t*>(src + j);
-    const uint32_t hi = *reinterpret_cast<const uint32_t*>(src + 64 + j);
-    const uint32_t wl = *reinterpret_cast<const uint32_t*>(w + j);
-    const uint32_t wh = *reinterpret_cast<const uint32_t*>(w + 64 + j);
-    float x[4] = {bf16_lo(lo), bf16_hi(lo), bf16_lo(hi), bf16_hi(hi)};
-    float ss = x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    const float r = rsqrtf(ss * (1.f / kHeadDim) + a.eps);
-    x[0] *= r * bf16_lo(wl);
-    x[1] *= r * bf16_hi(wl);
-    x[2] *= r * bf16_lo(wh);
-    x[3] *= r * bf16_hi(wh);
+    append_v(a, t);
+    if (node == node0 || pos != had) {
+      if (node != node0) __syncthreads();
+      if (threadIdx.x < kHeadDim / 2) {
+        Pair sn, cs;
+        sincos_pair(static_cast<double>(pos) * a.inv_freq[threadIdx.x], &sn, &cs);
+        s_cos[threadIdx.x] = cs.h + cs.l;
+        s_sin[threadIdx.x] = sn.h + sn.l;
+      }
+      __syncthreads();
+      had = pos;
+    }
     const float c0 = s_cos[j], s0 = s_sin[j], c1 = s_cos[j + 1], s1 = s_sin[j + 1];
-    const float y0 = x[0] * c0 - x[2] * s0, y1 = x[1] * c1 - x[3] * s1;   // dims j, j + 1
-    const float z0 = x[2] * c0 + x[0] * s0, z1 = x[3] * c1 + x[1] * s1;   // dims j + 64, j + 65
-    *reinterpret_cast<uint32_t*>(dst + j) = pack_bf16x2(y0, y1);
-    *reinterpret_cast<uint32_t*>(dst + 64 + j) = pack_bf16x2(z0, z1);
-  }
-  for (int w = threadIdx.x; w < a.hkv * 16; w += blockDim.x) {  // V: plain copy into the draft slot
-    const int kh = w >> 4, ch = w & 15;
-    const uint4 v = *reinterpret_cast<const uint4*>(
-        a.v_in + ((static_cast<size_t>(c) * a.n_new + i) * a.hkv + kh) * kHeadDim + ch * 8);
-    *reinterpret_cast<uint4*>(a.draft_v + ((static_cast<size_t>(c) * a.hkv + kh) * a.n_max + a.n0 + i) * kHeadDim +
-                              ch * 8) = v;
+    while (head < h1) {
+      __nv_bfloat16* dst =
+          head < a.hq ? a.q_out + (t.row * a.hq + head) * kHeadDim
+                      : a.draft_k + ((static_cast<size_t>(t.c) * a.hkv + head - a.hq) * a.n_max + a.n0 + t.i) * kHeadDim;
+      const __nv_bfloat16* w = head < a.hq ? a.q_norm_w : a.k_norm_w;
+      const uint32_t wl = *reinterpret_cast<const uint32_t*>(w + j);
+      const uint32_t wh = *reinterpret_cast<const uint32_t*>(w + 64 + j);
+      float x[4] = {bf16_lo(lo), bf16_hi(lo), bf16_lo(hi), bf16_hi(hi)};
+      head += kAppendThreads / 32;
+      if (head < h1) {  // the warp's next head
+        lo = *reinterpret_cast<const uint32_t*>(source(head));
+        hi = *reinterpret_cast<const uint32_t*>(source(head) + 64);
+      }
+      float ss = x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      const float r = rsqrtf(ss * (1.f / kHeadDim) + a.eps);
+      x[0] *= r * bf16_lo(wl);
+      x[1] *= r * bf16_hi(wl);
+      x[2] *= r * bf16_lo(wh);
+      x[3] *= r * bf16_hi(wh);
+      const float y0 = x[0] * c0 - x[2] * s0, y1 = x[1] * c1 - x[3] * s1;   // dims j, j + 1
+      const float z0 = x[2] * c0 + x[0] * s0, z1 = x[3] * c1 + x[1] * s1;   // dims j + 64, j + 65
+      *reinterpret_cast<uint32_t*>(dst + j) = pack_bf16x2(y0, y1);
+      *reinterpret_cast<uint32_t*>(dst + 64 + j) = pack_bf16x2(z0, z1);
+    }
   }
 }
 
@@ -272,12 +435,12 @@ cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream) {
   return cudaLaunchKernelEx(&cfg, merge_kernel, p);
 }
 
-cudaError_t launch_append(const AppendParams& a, cudaStream_t stream) {
-  if (a.q_norm_w != nullptr)
-    append_qknorm_kernel<<<a.C * a.n_new, kAppendThreads, 0, stream>>>(a);
-  else
-    append_kernel<<<a.C * a.n_new, kAppendThreads, 0, stream>>>(a);
-  return cudaGetLastError();
+cudaError_t launch_append(AppendParams a, cudaStream_t stream) {
+  const int nodes = a.C * a.n_new;
+  const int splits = std::max(1, std::min(kAppendSplits, kAppendCtas / nodes));
+  a.group = std::max(1, std::min(kAppendGroup, nodes / kAppendCtas));
+  return launch_maybe_pdl(a.q_norm_w != nullptr ? append_qknorm_kernel : append_kernel,
+                          dim3((nodes + a.group - 1) / a.group, splits), dim3(kAppendThreads), 0, true, stream, a);
 }
 
 }  // namespace kvshot
