@@ -384,14 +384,15 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
     prefetch_tensormap(&maps.dv);
   }
   build_plan(p, sm.len, sm.base);
-  // With KVSHOT_OVERLAP_PREVIOUS the kernel may have started before the preceding kernel ended:
-  // q and the draft K/V (and every output) are touched only after it has.
-  wait_for_prerequisite_grid();
   const Cursor cu = cursor_begin(p, sm.len, sm.base);
   Pipe pipe{sm.ring, sm.full, sm.empty, CF::kStages, reinterpret_cast<volatile int*>(&sm.misc[0]), &sm.misc[1]};
   if (warp == CF::kWarps) {
     run_producer(p, maps, pipe, sm.len, cu);
   } else {
+    // With KVSHOT_OVERLAP_PREVIOUS the kernel may have started before the preceding kernel ended: the
+    // producer loads target tiles meanwhile (draft tiles after it); q is read, and outputs are written,
+    // only once it has.
+    wait_for_prerequisite_grid();
     run_consumer<CF>(p, sm, pipe, cu);
   }
   __syncthreads();

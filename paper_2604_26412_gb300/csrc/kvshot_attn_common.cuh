@@ -499,6 +499,7 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
   uint32_t phase = 0;
   int issued = 0;
   int piece = 0;
+  bool waited = false;  // griddepcontrol.wait done
   PageWindow win;
   while (cu.t < cu.t_end) {
     const int h = cu.hr / p.row_blocks;
@@ -506,6 +507,10 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
     const bool draft = cu.lt >= cu.pt;
     const int key0 = (draft ? cu.lt - cu.pt : cu.lt) * kTileKeys;
     const int nkeys = min(kTileKeys, (draft ? p.N : L) - key0);
+    if (draft && !waited) {  // the draft K/V may come from the preceding kernel (KVSHOT_OVERLAP_PREVIOUS)
+      wait_for_prerequisite_grid();
+      waited = true;
+    }
     // Page ids of this tile's boxes (box i covers rows key0 + i * box_rows).
     int pids[kTileKeys / 8];
     if (p.paged && !draft) {
