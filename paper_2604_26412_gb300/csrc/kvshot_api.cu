@@ -475,6 +475,10 @@ extern "C" kvshot_status kvshot_draft_attn(const kvshot_attn_desc* d, const void
                   : pl.kernel == Kernel::kTensorMemory ? launch_attn_tc(p, maps, pl.nq_box, pl.spread, pl.pair, pdl, s)
                                                        : launch_attn_cc(p, maps, pdl, s);
   if (e != cudaSuccess) return KVSHOT_ERR_CUDA;
+  // One cache whose units divide evenly over the CTAs: every CTA takes whole units whatever the length, and
+  // nothing is left to merge (tiny chain: one launch of three).
+  const int cache_units = d->hkv * pl.row_blocks;
+  if (pl.num_ctas == 1 || (d->num_caches == 1 && cache_units % pl.num_ctas == 0)) return KVSHOT_OK;
   e = launch_merge(p, s);
   return e == cudaSuccess ? KVSHOT_OK : KVSHOT_ERR_CUDA;
 }

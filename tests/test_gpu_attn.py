@@ -110,6 +110,19 @@ def test_forced_kernels_agree_with_oracle(flags, nq):
         gh.compare(out, lse, ref_out, ref_lse, f"flags={flags} nq={nq}")
 
 
+# One cache: grids that divide its units run without the merge kernel, the others with it, at every length.
+@pytest.mark.parametrize("num_ctas", [1, 2, 3, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("length", [0, 1, 200, 640])
+def test_one_cache_with_and_without_merge(length, num_ctas):
+    spec, inp, dk, dv, q, N, Nq = _case((640,), (2, 3), True, True, 16, 32, 8, 3, seed=9)
+    inp.seq_lens.fill_(length)
+    hc = gh.HostCache(inp)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for flags in (0, kvshot.KVSHOT_FORCE_MMA, kvshot.KVSHOT_FORCE_TC, kvshot.KVSHOT_FORCE_CC):
+        out, lse = _run(spec, inp, dk, dv, q, N, Nq, flags=flags, num_ctas=num_ctas)
+        gh.compare(out, lse, ref_out, ref_lse, f"L={length} flags={flags} ctas={num_ctas}")
+
+
 def test_scale_parameter():
     spec, inp, dk, dv, q, N, Nq = _case((150,), (2, 2), True, True, 16, 32, 8, 2, seed=5)
     hc = gh.HostCache(inp)
