@@ -182,8 +182,7 @@ extern "C" kvshot_status kvshot_kv_project(const kvshot_project_desc* d, const v
   p.num_pages = paged ? d->num_pages : 0;
   p.l_cap = paged ? 0 : d->l_cap;
   p.rope = (d->flags & KVSHOT_PROJECT_ROPE) ? 1 : 0;
-  for (int j = 0; j < kHeadDim / 2; ++j)
-    p.inv_freq[j] = std::pow(static_cast<double>(d->rope_base), -2.0 * j / kHeadDim);
+  rope_frequencies(d->rope_base, p.inv_freq);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -135,6 +135,17 @@ bool encode_bf16_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+void rope_frequencies(float rope_base, double* inv_freq) {
+  static thread_local float base = 0.f;  // rope_base > 0
+  static thread_local double table[kHeadDim / 2];
+  if (base != rope_base) {
+    for (int j = 0; j < kHeadDim / 2; ++j)
+      table[j] = std::pow(static_cast<double>(rope_base), -2.0 * j / kHeadDim);
+    base = rope_base;
+  }
+  std::copy(table, table + kHeadDim / 2, inv_freq);
+}
+
 namespace {
 
 // 4-D view {128 dims, hq, Nq, C} of q [C, Nq, hq, 128]; a box is one 64-dim
@@ -178,6 +189,30 @@ int sm_count() {
   if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   if (dev >= 0 && dev < 64) cached[dev] = n;
   return n;
+}
+
+// CTAs per SM of a plan's kernel: a property of the device, the kernel and its shared memory (so of the number
+// of caches), asked of the runtime once per thread and then kept (one entry: a program's calls mostly agree).
+cudaError_t ctas_per_sm(Kernel kernel, int m_tiles, int rows_per_unit, int C, int* per_sm) {
+  struct Known {
+    int dev = -1, kernel, m_tiles, rows, C, per_sm;
+  };
+  static thread_local Known k;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (k.dev != dev || k.kernel != static_cast<int>(kernel) || k.m_tiles != m_tiles || k.rows != rows_per_unit ||
+      k.C != C) {
+    int n = 0;
+    e = kernel == Kernel::kMma            ? attn_mma_occupancy(m_tiles, C, &n)
+        : kernel == Kernel::kMmaF8        ? attn_f8_occupancy(rows_per_unit, C, &n)
+        : kernel == Kernel::kTensorMemory ? attn_tc_occupancy(C, &n)
+                                          : attn_cc_occupancy(C, &n);
+    if (e != cudaSuccess) return e;
+    k.dev = dev, k.kernel = static_cast<int>(kernel), k.m_tiles = m_tiles, k.rows = rows_per_unit, k.C = C, k.per_sm = n;
+  }
+  *per_sm = k.per_sm;
+  return cudaSuccess;
 }
 
 // Checks that do not depend on the cache layout.
@@ -299,10 +334,7 @@ kvshot_status make_plan_for(const kvshot_attn_desc* d, bool paged, bool small_bl
   int grid = d->num_ctas;
   if (grid == 0) {
     int per_sm = 0;
-    const cudaError_t e = pl->kernel == Kernel::kMma ? attn_mma_occupancy(pl->m_tiles, d->num_caches, &per_sm)
-                          : pl->kernel == Kernel::kMmaF8 ? attn_f8_occupancy(pl->rows_per_unit, d->num_caches, &per_sm)
-                          : pl->kernel == Kernel::kTensorMemory ? attn_tc_occupancy(d->num_caches, &per_sm)
-                                                                 : attn_cc_occupancy(d->num_caches, &per_sm);
+    const cudaError_t e = ctas_per_sm(pl->kernel, pl->m_tiles, pl->rows_per_unit, d->num_caches, &per_sm);
     const int sms = sm_count();
     if (e != cudaSuccess || per_sm < 1 || sms < 1) return KVSHOT_ERR_CUDA;
     grid = sms * per_sm;
@@ -520,8 +552,7 @@ kvshot_status draft_append(const kvshot_attn_desc* d, const void* q_in, const vo
   ap.n_max = d->n_max;
   ap.n0 = n0;
   ap.n_new = n_new;
-  for (int j = 0; j < kHeadDim / 2; ++j)
-    ap.inv_freq[j] = std::pow(static_cast<double>(rope_base), -2.0 * j / kHeadDim);
+  rope_frequencies(rope_base, ap.inv_freq);
   ap.q_norm_w = static_cast<const __nv_bfloat16*>(q_norm_w);
   ap.k_norm_w = static_cast<const __nv_bfloat16*>(k_norm_w);
   ap.eps = eps;

@@ -117,6 +117,10 @@ struct TensorMaps {
 bool encode_bf16_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                     uint32_t box_rows);
 
+// inv_freq[j] = rope_base^(-2j/128), j in [0, 64).  Each thread keeps the table of its last rope_base (64 pow calls
+// are ~1.3 us of a call's host time).
+void rope_frequencies(float rope_base, double* inv_freq);
+
 // Kernel launchers (one per translation unit).  Return cudaSuccess or the launch error.  `pdl`:
 // launch with programmatic stream serialization (KVSHOT_OVERLAP_PREVIOUS).
 cudaError_t launch_attn_cc(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream);

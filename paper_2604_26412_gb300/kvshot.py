@@ -164,7 +164,17 @@ def version() -> int:
     return int(load().kvshot_version())
 
 
+# Marshalling is on the critical path of short drafting steps (a level of a small chain takes ~10 us on the
+# GPU), so the calls below test for the usual types first and make no intermediate objects: 12 arguments cost
+# ~2 us instead of ~6.
+_Tensor = torch.Tensor
+_getdevice = getattr(torch._C, "_cuda_getDevice", None)
+_rawstream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _ptr(x) -> Optional[int]:
+    if type(x) is _Tensor:
+        return x.data_ptr()
     if x is None:
         return None
     if isinstance(x, int):
@@ -180,7 +190,11 @@ def _dref(desc):
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        if _rawstream is not None and _getdevice is not None and torch.cuda.is_initialized():
+            return _rawstream(_getdevice())  # the current stream's handle, without a Stream object
         return torch.cuda.current_stream().cuda_stream
+    if type(stream) is int:
+        return stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
@@ -203,9 +217,9 @@ def workspace_size(desc: AttnDesc) -> int:
 def draft_attn_status(desc: AttnDesc, q, target_k, target_v, page_table, seq_lens, draft_k, draft_v, tree_parent, out,
                       lse, stream=None) -> int:
     """Call kvshot_draft_attn and return its status code."""
-    return int(load().kvshot_draft_attn(_dref(desc), _ptr(q), _ptr(target_k), _ptr(target_v),
+    return (_lib or load()).kvshot_draft_attn(_dref(desc), _ptr(q), _ptr(target_k), _ptr(target_v),
                                         _ptr(page_table), _ptr(seq_lens), _ptr(draft_k), _ptr(draft_v),
-                                        _ptr(tree_parent), _ptr(out), _ptr(lse), _stream(stream)))
+                                        _ptr(tree_parent), _ptr(out), _ptr(lse), _stream(stream))
 
 
 def draft_attn(desc: AttnDesc, q, target_k, target_v, page_table, seq_lens, draft_k, draft_v, tree_parent, out, lse,
@@ -219,16 +233,16 @@ def draft_attn(desc: AttnDesc, q, target_k, target_v, page_table, seq_lens, draf
 def draft_attn_static_status(desc: AttnDesc, q, target_k, target_v, page_table, seq_lens, draft_k, draft_v,
                              tree_parent, out, lse, stream=None) -> int:
     """Call kvshot_draft_attn_static (library-owned scratch, no allocation) and return its status."""
-    return int(load().kvshot_draft_attn_static(_dref(desc), _ptr(q), _ptr(target_k), _ptr(target_v),
+    return (_lib or load()).kvshot_draft_attn_static(_dref(desc), _ptr(q), _ptr(target_k), _ptr(target_v),
                                                _ptr(page_table), _ptr(seq_lens), _ptr(draft_k), _ptr(draft_v),
-                                               _ptr(tree_parent), _ptr(out), _ptr(lse), _stream(stream)))
+                                               _ptr(tree_parent), _ptr(out), _ptr(lse), _stream(stream))
 
 
 def draft_append_status(desc: AttnDesc, q_in, k_in, v_in, positions, n0: int, n_new: int, rope_base: float, draft_k,
                         draft_v, q_out, stream=None) -> int:
-    return int(load().kvshot_draft_append(_dref(desc), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(positions),
+    return (_lib or load()).kvshot_draft_append(_dref(desc), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(positions),
                                           int(n0), int(n_new), float(rope_base), _ptr(draft_k), _ptr(draft_v),
-                                          _ptr(q_out), _stream(stream)))
+                                          _ptr(q_out), _stream(stream))
 
 
 def draft_append(desc: AttnDesc, q_in, k_in, v_in, positions, n0: int, n_new: int, rope_base: float, draft_k, draft_v,
@@ -248,8 +262,8 @@ def gated_delta_workspace_size(desc: FusionDesc) -> int:
 
 def gated_delta_status(desc: FusionDesc, n, o, w_g, b_g, w_delta, h, stream=None) -> int:
     """Call kvshot_gated_delta (h = n + sigmoid(W_g [n; o; o - n] + b_g) * W_delta (o - n)); return its status."""
-    return int(load().kvshot_gated_delta(_dref(desc), _ptr(n), _ptr(o), _ptr(w_g), _ptr(b_g), _ptr(w_delta),
-                                         _ptr(h), _stream(stream)))
+    return (_lib or load()).kvshot_gated_delta(_dref(desc), _ptr(n), _ptr(o), _ptr(w_g), _ptr(b_g), _ptr(w_delta),
+                                         _ptr(h), _stream(stream))
 
 
 def gated_delta(desc: FusionDesc, n, o, w_g, b_g, w_delta, h, stream=None) -> None:
@@ -273,8 +287,8 @@ def kv_project_workspace_size(desc: ProjectDesc) -> int:
 def kv_project_status(desc: ProjectDesc, k_in, v_in, w_k, w_v, token_cache, positions, page_table, k_out, v_out,
                       stream=None) -> int:
     """Call kvshot_kv_project (K' = W_K [K_1..K_L] (+ RoPE), V' = W_V [V_1..V_L] into the reused cache)."""
-    return int(load().kvshot_kv_project(_dref(desc), _ptr(k_in), _ptr(v_in), _ptr(w_k), _ptr(w_v), _ptr(token_cache),
-                                        _ptr(positions), _ptr(page_table), _ptr(k_out), _ptr(v_out), _stream(stream)))
+    return (_lib or load()).kvshot_kv_project(_dref(desc), _ptr(k_in), _ptr(v_in), _ptr(w_k), _ptr(w_v), _ptr(token_cache),
+                                        _ptr(positions), _ptr(page_table), _ptr(k_out), _ptr(v_out), _stream(stream))
 
 
 def kv_project(desc: ProjectDesc, k_in, v_in, w_k, w_v, token_cache, positions, page_table, k_out, v_out,
@@ -286,10 +300,10 @@ def kv_project(desc: ProjectDesc, k_in, v_in, w_k, w_v, token_cache, positions, 
 
 def draft_append_qknorm_status(desc: AttnDesc, q_in, k_in, v_in, positions, n0: int, n_new: int, rope_base: float,
                                q_norm_w, k_norm_w, eps: float, draft_k, draft_v, q_out, stream=None) -> int:
-    return int(load().kvshot_draft_append_qknorm(_dref(desc), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(positions),
+    return (_lib or load()).kvshot_draft_append_qknorm(_dref(desc), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(positions),
                                                  int(n0), int(n_new), float(rope_base), _ptr(q_norm_w),
                                                  _ptr(k_norm_w), float(eps), _ptr(draft_k), _ptr(draft_v),
-                                                 _ptr(q_out), _stream(stream)))
+                                                 _ptr(q_out), _stream(stream))
 
 
 def draft_append_qknorm(desc: AttnDesc, q_in, k_in, v_in, positions, n0: int, n_new: int, rope_base: float, q_norm_w,

@@ -86,6 +86,7 @@ class DraftStep:
 
     def run(self, stream: Optional[torch.cuda.Stream] = None) -> None:
         inp = self.inp
+        stream = kvshot._stream(stream)  # once for all calls
         n0 = 0
         for i, n_step in enumerate(self.levels):
             d = self.descs[i]
