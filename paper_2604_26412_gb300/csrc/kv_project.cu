@@ -13,89 +13,265 @@
 // (App. B: verified prefix positions take the target's -- here projected --
 // K/V), so the cache is built incrementally, a few tokens per decoding step.
 //
-// Two kernels.  The slab GEMM (kvshot_slab_gemm.cuh) computes the products per
-// layer block (table entry (K or V, layer l): W[:, l d_kv : (l+1) d_kv] times
-// the tokens' layer-l K or V), into fp32 slabs [2 L_s][T][d_kv].
-// kv_project_finish adds each output's L_s slabs, rotates the keys, rounds to
-// bf16 and stores both vectors into the cache through the page table.  The
-// angle pos * rope_base^(-2j/128) is formed and reduced modulo 2 pi in fp64
-// (from a host table of the frequencies); sine, cosine and the rotation are
-// fp32 (relative error ~1e-7, far below the bf16 rounding that follows).
-// fp64 sine and cosine cost this latency-bound kernel ~2 us per call on GB300.
+// One kernel.  A cluster of up to 8 CTAs owns the 128 output features of one KV head (K or V) for a block of up
+// to 128 tokens and splits the L_s d_kv inputs among its CTAs: each runs its part of the GEMM on the tcgen05
+// tensor cores (weights as A, tokens as B, fp32 accumulator in tensor memory), leaves its partial sums in its
+// shared memory, and after a cluster barrier adds the cluster's partials (in rank order) for its share of the
+// tokens, rotates the keys, rounds to bf16 and stores both halves of the head into the cache through the page table.
+// What bounds it: the weights' bytes (one decoding step's few tokens, 2 L_s d_kv^2 bf16 values; an SM ingests
+// ~44 KB/us) and the fixed latencies of launch, load, MMA and exchange, which slot and angle look-ups overlap.
+// Measured, 4 layers of 8 heads, back to back in a graph: 1 token 6.7 us, 32 tokens 7.7, 512 tokens 20.4 us; as a
+// GEMM into fp32 slabs per layer and a second kernel to add them 11.8, 12.5 and 21.5 us.
+// The angle pos * rope_base^(-2j/128) is formed and reduced modulo 2 pi in fp64 (from a host table of the
+// frequencies); sine, cosine and the rotation are fp32 (relative error ~1e-7, far below the bf16 rounding that
+// follows).  fp64 sine and cosine cost this latency-bound kernel ~2 us per call on GB300.
 #include <algorithm>
 #include <cmath>
 
-#include "kvshot_slab_gemm.cuh"
+#include "kvshot_attn_common.cuh"
+#include "kvshot_tcgen05.cuh"
 
 namespace kvshot {
 namespace {
 
 using namespace dev;
+using namespace tc;
 
-constexpr int kFinishThreads = 256;  // (token, KV head) pairs of 64 rotation pairs: 4 per CTA
-constexpr int kMaxLayers = sg::kMaxEntries / 2;
+constexpr int kMaxLayers = 8;
+constexpr int kThreads = 256;
+constexpr int kFeat = kHeadDim;              // output features per cluster (MMA M): one KV head
+constexpr int kTok = 128;                    // most tokens per cluster (MMA N)
+constexpr int kKT = 64;                      // inputs per k-tile: one 128-byte swizzled row
+constexpr int kABytes = kFeat * kKT * 2;     // a k-tile of weights
+// Two CTAs fit an SM: with one (a ring of 192 KB) only 15 clusters of 8 are resident at a time, and the 16 of an
+// 8-head cache took a second wave (12.9 against 8.1 us per call, 32 tokens of 4 layers).
+constexpr int kRingBytes = 102 * 1024;
+constexpr int kMaxStages = 5;
+constexpr int kMaxSplit = 8;                 // CTAs per cluster (the portable limit)
+constexpr int kProjectCtas = 288;            // CTAs of 8-CTA clusters resident at a time
 
 struct ProjectParams {
-  const float* slab;  // [2 L][T][d_kv]
   const int32_t* token_cache;
   const int32_t* positions;
   const int32_t* page_table;  // null: contiguous cache
   __nv_bfloat16* k_out;
   __nv_bfloat16* v_out;
   int32_t* err;
-  int T, L, hkv, C;
+  int T, hkv, C;
+  int nk;       // k-tiles: L d_kv / 64
+  int box_tok;  // tokens per cluster: min(T, kTok)
+  int split;    // CTAs per cluster
+  int stages;   // ring slots of a k-tile of weights and one of tokens
   int paged, page_size, max_pages, num_pages, l_cap;
   int rope;
   double inv_freq[kHeadDim / 2];  // rope_base^(-2j/128), fp64
 };
 
-// One thread per (token, KV head, rotation pair j in [0, 64)): features j and j + 64 of the head.
-__global__ void __launch_bounds__(kFinishThreads) kv_project_finish(const __grid_constant__ ProjectParams p) {
-  wait_for_prerequisite_grid();
-  const int dkv = p.hkv * kHeadDim;
-  const int g = blockIdx.x * (kFinishThreads / 64) + (threadIdx.x >> 6);  // (token, head)
-  const int j = threadIdx.x & 63;
-  if (g >= p.T * p.hkv) return;
-  const int t = g / p.hkv, h = g - t * p.hkv;
-  const int c = p.token_cache[t], pos = p.positions[t];
-  const int cap = p.paged ? p.max_pages * p.page_size : p.l_cap;
-  if (c < 0 || c >= p.C || pos < 0 || pos >= cap) {
-    if (j == 0) set_error(p.err, KVSHOT_ERR_DEVICE_BOUNDS);
-    return;
-  }
+// Maps: weights [d_kv, L d_kv] of K and V, boxes {64, 128}; tokens [T, L d_kv], boxes {64, box_tok}.
+struct ProjectMaps {
+  CUtensorMap w[2], a[2];
+};
+
+__host__ __device__ inline int mma_n(int box_tok) { return (box_tok + 15) / 16 * 16; }
+__host__ __device__ inline int slot_bytes(int box_tok) { return kABytes + mma_n(box_tok) * kKT * 2; }
+
+// Shared memory: the ring, later the partial sums [tokens][128] fp32; then the barriers.
+__host__ __device__ inline size_t ring_bytes(int stages, int box_tok) {
+  const size_t ring = static_cast<size_t>(stages) * slot_bytes(box_tok);
+  const size_t sums = static_cast<size_t>(mma_n(box_tok) + 31) / 32 * 32 * kFeat * 4;
+  return ring > sums ? ring : sums;
+}
+inline size_t smem_bytes(int stages, int box_tok) {
+  return 1024 + (ring_bytes(stages, box_tok) + 1023) / 1024 * 1024 + 8 * (2 * kMaxStages + 1) + 16;
+}
+
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
+          "r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Two floats from the shared memory of CTA `rank` of the cluster, at this CTA's address `addr`.
+__device__ __forceinline__ float2 cluster_load(uint32_t addr, int rank) {
+  float2 v;
+  asm volatile(
+      "{\n\t.reg .u32 ra;\n\tmapa.shared::cluster.u32 ra, %2, %3;\n\t"
+      "ld.shared::cluster.v2.f32 {%0, %1}, [ra];\n\t}"
+      : "=f"(v.x), "=f"(v.y)
+      : "r"(addr), "r"(rank)
+      : "memory");
+  return v;
+}
+
+// Where a token's head goes, and the angles of its pairs (j, j + 64) and (j + 1, j + 65).
+struct Slot {
+  bool in;  // the cache, position and page id are in range
   size_t row;
-  if (p.paged) {
-    const int pid = p.page_table[static_cast<size_t>(c) * p.max_pages + pos / p.page_size];
-    if (pid < 0 || pid >= p.num_pages) {
-      if (j == 0) set_error(p.err, KVSHOT_ERR_DEVICE_BOUNDS);
-      return;
+  float2 cs, sn;
+};
+__device__ __forceinline__ Slot find_slot(const ProjectParams& p, int tok, int h, int j, int kv) {
+  Slot s;
+  const int c = p.token_cache[tok], pos = p.positions[tok];
+  const int cap = p.paged ? p.max_pages * p.page_size : p.l_cap;
+  s.in = c >= 0 && c < p.C && pos >= 0 && pos < cap;
+  s.row = 0;
+  if (s.in) {
+    if (p.paged) {
+      const int pid = p.page_table[static_cast<size_t>(c) * p.max_pages + pos / p.page_size];
+      s.in = pid >= 0 && pid < p.num_pages;
+      s.row = (static_cast<size_t>(pid) * p.hkv + h) * p.page_size + pos % p.page_size;
+    } else {
+      s.row = (static_cast<size_t>(c) * p.hkv + h) * p.l_cap + pos;
     }
-    row = (static_cast<size_t>(pid) * p.hkv + h) * p.page_size + pos % p.page_size;
-  } else {
-    row = (static_cast<size_t>(c) * p.hkv + h) * p.l_cap + pos;
   }
-  const size_t td = static_cast<size_t>(p.T) * dkv;
-  const size_t f = static_cast<size_t>(t) * dkv + h * kHeadDim + j;
-  float kx = 0.f, ky = 0.f, vx = 0.f, vy = 0.f;
-  for (int l = 0; l < p.L; ++l) {
-    kx += p.slab[l * td + f];
-    ky += p.slab[l * td + f + 64];
-    vx += p.slab[(p.L + l) * td + f];
-    vy += p.slab[(p.L + l) * td + f + 64];
+  s.cs = s.sn = make_float2(0.f, 0.f);
+  if (p.rope && kv == 0) {
+    float r[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const double a = static_cast<double>(pos) * p.inv_freq[j + e];
+      r[e] = static_cast<float>(a - 6.283185307179586 * rint(a * 0.15915494309189535));
+    }
+    sincosf(r[0], &s.sn.x, &s.cs.x);
+    sincosf(r[1], &s.sn.y, &s.cs.y);
   }
-  if (p.rope) {
-    const double a = static_cast<double>(pos) * p.inv_freq[j];
-    const double r = a - 6.283185307179586 * rint(a * 0.15915494309189535);
-    float sn, cs;
-    sincosf(static_cast<float>(r), &sn, &cs);
-    const float x = kx, y = ky;
-    kx = x * cs - y * sn;
-    ky = y * cs + x * sn;
+  return s;
+}
+
+// Grid (token block x cluster rank, KV head, (0: K, 1: V)).
+__global__ void __launch_bounds__(kThreads, 1)
+    kv_project_kernel(const __grid_constant__ ProjectParams p, const __grid_constant__ ProjectMaps maps) {
+  extern __shared__ uint8_t smem_raw[];
+  const int split = p.split, tb = blockIdx.x / split, rank = blockIdx.x - tb * split, h = blockIdx.y, kv = blockIdx.z;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int N = mma_n(p.box_tok), slot = slot_bytes(p.box_tok);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + (ring_bytes(p.stages, p.box_tok) + 1023) / 1024 * 1024);
+  uint64_t* empty = full + kMaxStages;
+  uint64_t* done = empty + kMaxStages;
+  uint32_t* tmem_base = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* gave_up = reinterpret_cast<volatile int*>(tmem_base + 1);  // a wait timed out
+  const int k0 = p.nk * rank / split, n = p.nk * (rank + 1) / split - k0;  // this CTA's k-tiles
+  const uint32_t cols = N <= 32 ? 32u : N <= 64 ? 64u : 128u;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(smem_addr(&full[s]), 1);
+      mbar_init(smem_addr(&empty[s]), 1);
+    }
+    mbar_init(smem_addr(done), 1);
+    *gave_up = 0;
+    fence_mbar_init();
+    prefetch_tensormap(&maps.w[kv]);
+    prefetch_tensormap(&maps.a[kv]);
   }
-  p.k_out[row * kHeadDim + j] = __float2bfloat16_rn(kx);
-  p.k_out[row * kHeadDim + j + 64] = __float2bfloat16_rn(ky);
-  p.v_out[row * kHeadDim + j] = __float2bfloat16_rn(vx);
-  p.v_out[row * kHeadDim + j + 64] = __float2bfloat16_rn(vy);
+  if (warp == 1) {
+    tmem_alloc(smem_addr(tmem_base), cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_base;
+  wait_for_prerequisite_grid();  // launched behind the preceding kernel: nothing before this touches its results
+  if (threadIdx.x == 0) allow_dependent_launch();
+  bool ok = true;
+  int issued = 0;
+  if (warp == 0 && lane == 0) {
+    for (int kt = 0; kt < n; ++kt) {
+      const int s = kt % p.stages;
+      if (kt >= p.stages) ok = mbar_wait(smem_addr(&empty[s]), (kt / p.stages - 1) & 1, p.err);
+      if (!ok) break;
+      const uint32_t bar = smem_addr(&full[s]), dst = smem_addr(base + s * slot);
+      mbar_arrive_expect_tx(bar, kABytes + p.box_tok * kKT * 2);
+      tma_load(dst, &maps.w[kv], (k0 + kt) * kKT, h * kFeat, bar);
+      tma_load(dst + kABytes, &maps.a[kv], (k0 + kt) * kKT, tb * p.box_tok, bar);
+      issued = kt + 1;
+    }
+    if (!ok) *gave_up = 1;
+  }
+  __syncwarp();
+  // This CTA's share of the tokens, a warp per token: lane l has pairs (j, j + 64), j = 2 l and 2 l + 1.  The slot
+  // and the angles of a warp's first token are looked up while the loads are in flight.
+  const int tokens = min(p.box_tok, p.T - tb * p.box_tok);
+  const int t0 = tokens * rank / split + warp, t1 = tokens * (rank + 1) / split, j = 2 * lane;
+  Slot place{};
+  if (t0 < t1) place = find_slot(p, tb * p.box_tok + t0, h, j, kv);
+  if (warp == 1 && lane == 0) {
+    const uint32_t idesc = idesc_bf16(kFeat, N, false);
+    for (int kt = 0; kt < n; ++kt) {
+      const int s = kt % p.stages;
+      ok = mbar_wait(smem_addr(&full[s]), (kt / p.stages) & 1, p.err);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t a0 = smem_addr(base + s * slot), b0 = a0 + kABytes;
+#pragma unroll
+      for (int ks = 0; ks < kKT / 16; ++ks)
+        tc_mma(tmem, smem_desc_sw128(a0 + ks * 32, 16, 1024), smem_desc_sw128(b0 + ks * 32, 16, 1024), idesc,
+               (kt | ks) ? 1u : 0u);
+      if (kt + p.stages < n) tc_commit(smem_addr(&empty[s]));
+    }
+    if (!ok) *gave_up = 1;
+    tc_commit(smem_addr(done));  // every MMA this thread issued has completed
+  }
+  __syncwarp();
+  mbar_wait(smem_addr(done), 0, p.err);
+  tc_fence_after();
+  if (threadIdx.x == 0 && *gave_up)  // let the copies in flight land before their memory is used again
+    for (int kt = max(0, issued - p.stages); kt < issued; ++kt)
+      mbar_wait(smem_addr(&full[kt % p.stages]), (kt / p.stages) & 1, p.err);
+  // Partial sums to shared memory, [token][feature], over the ring (every load has been consumed).
+  float* sums = reinterpret_cast<float*>(base);
+  const int quarter = warp & 3;  // of the TMEM lanes (features); the two warpgroups take alternate chunks of tokens
+  const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+#pragma unroll 1
+  for (int c = warp >> 2; c * 32 < tokens; c += kThreads / 128) {
+    uint32_t x[32];
+    tmem_ld32(trow + c * 32, x);
+    tmem_wait_ld();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) sums[(c * 32 + j) * kFeat + quarter * 32 + lane] = __uint_as_float(x[j]);
+  }
+  tc_fence_before();
+  cluster_sync();
+  if (warp == 1) tmem_dealloc(tmem, cols);
+  Slot next = place;
+  for (int t = t0; t < t1; t += kThreads / 32) {
+    place = next;
+    if (t + kThreads / 32 < t1) next = find_slot(p, tb * p.box_tok + t + kThreads / 32, h, j, kv);
+    const uint32_t at = smem_addr(sums + t * kFeat + j);
+    float2 a[kMaxSplit], b[kMaxSplit];
+#pragma unroll
+    for (int r = 0; r < kMaxSplit; ++r) {  // every load goes out before the first sum
+      a[r] = r < split ? cluster_load(at, r) : make_float2(0.f, 0.f);
+      b[r] = r < split ? cluster_load(at + 64 * 4, r) : make_float2(0.f, 0.f);
+    }
+    float2 lo = a[0], hi = b[0];
+#pragma unroll
+    for (int r = 1; r < kMaxSplit; ++r) {
+      lo.x += a[r].x;
+      lo.y += a[r].y;
+      hi.x += b[r].x;
+      hi.y += b[r].y;
+    }
+    if (!place.in) {
+      if (lane == 0) set_error(p.err, KVSHOT_ERR_DEVICE_BOUNDS);
+      continue;
+    }
+    if (p.rope && kv == 0) {
+      const float2 x = lo, y = hi;
+      lo = make_float2(x.x * place.cs.x - y.x * place.sn.x, x.y * place.cs.y - y.y * place.sn.y);
+      hi = make_float2(y.x * place.cs.x + x.x * place.sn.x, y.y * place.cs.y + x.y * place.sn.y);
+    }
+    __nv_bfloat16* out = (kv ? p.v_out : p.k_out) + place.row * kHeadDim + j;
+    *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(lo.x, lo.y);
+    *reinterpret_cast<uint32_t*>(out + 64) = pack_bf16x2(hi.x, hi.y);
+  }
+  cluster_sync();  // the partial sums are read by the other CTAs until here
 }
 
 bool aligned(const void* ptr, size_t a) { return (reinterpret_cast<uintptr_t>(ptr) % a) == 0; }
@@ -144,28 +320,7 @@ extern "C" kvshot_status kvshot_kv_project(const kvshot_project_desc* d, const v
   if (d->workspace == nullptr || !aligned(d->workspace, 256) || d->workspace_bytes < slab_bytes(d))
     return KVSHOT_ERR_WORKSPACE;
   const int T = d->num_tokens, L = d->num_layers, dkv = d->hkv * kHeadDim;
-  sg::Params gp;
-  gp.slab = static_cast<float*>(d->workspace);
-  gp.err = d->err_flag;
-  gp.T = T;
-  gp.d_out = dkv;
-  gp.box_tok = std::min(T, sg::kMaxTok);
-  // weight maps: 0 = W_K, 1 = W_V; activation maps: 0 = K of the L layers, 1 = V ([T, L d_kv] rows)
-  for (int l = 0; l < L; ++l) {
-    gp.e[l] = sg::Entry{0, 0, -1, 0, l * dkv, l * dkv, dkv / sg::kKT};
-    gp.e[L + l] = sg::Entry{1, 1, -1, 0, l * dkv, l * dkv, dkv / sg::kKT};
-  }
-  const uint64_t K = static_cast<uint64_t>(L) * dkv;
-  sg::Maps maps;
-  if (!encode_bf16_2d(&maps.w[0], w_k, K, dkv, sg::kKT, sg::kFeat) ||
-      !encode_bf16_2d(&maps.w[1], w_v, K, dkv, sg::kKT, sg::kFeat) ||
-      !encode_bf16_2d(&maps.a[0], k_in, K, T, sg::kKT, static_cast<uint32_t>(gp.box_tok)) ||
-      !encode_bf16_2d(&maps.a[1], v_in, K, T, sg::kKT, static_cast<uint32_t>(gp.box_tok)))
-    return KVSHOT_ERR_CUDA;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (sg::launch(gp, maps, 2 * L, s) != cudaSuccess) return KVSHOT_ERR_CUDA;
   ProjectParams p;
-  p.slab = gp.slab;
   p.token_cache = token_cache;
   p.positions = positions;
   p.page_table = page_table;
@@ -173,9 +328,10 @@ extern "C" kvshot_status kvshot_kv_project(const kvshot_project_desc* d, const v
   p.v_out = static_cast<__nv_bfloat16*>(v_out);
   p.err = d->err_flag;
   p.T = T;
-  p.L = L;
   p.hkv = d->hkv;
   p.C = d->num_caches;
+  p.nk = L * dkv / kKT;
+  p.box_tok = std::min(T, kTok);
   p.paged = paged ? 1 : 0;
   p.page_size = paged ? d->page_size : 0;
   p.max_pages = paged ? d->max_pages_per_seq : 0;
@@ -183,15 +339,36 @@ extern "C" kvshot_status kvshot_kv_project(const kvshot_project_desc* d, const v
   p.l_cap = paged ? 0 : d->l_cap;
   p.rope = (d->flags & KVSHOT_PROJECT_ROPE) ? 1 : 0;
   rope_frequencies(d->rope_base, p.inv_freq);
-  cudaLaunchAttribute attr[1];
+  // As many CTAs per cluster as keep the grid within one wave (a k-tile each at least).
+  const int blocks = (T + p.box_tok - 1) / p.box_tok;
+  const int64_t clusters = static_cast<int64_t>(2) * d->hkv * blocks;
+  int split = kMaxSplit;
+  while (split > 1 && (clusters * split > kProjectCtas || split > p.nk)) split /= 2;
+  p.split = split;
+  const int per_cta = (p.nk + split - 1) / split;
+  p.stages = std::min({per_cta, kMaxStages, kRingBytes / slot_bytes(p.box_tok)});
+  const uint64_t K = static_cast<uint64_t>(L) * dkv;
+  ProjectMaps maps;
+  if (!encode_bf16_2d(&maps.w[0], w_k, K, dkv, kKT, kFeat) || !encode_bf16_2d(&maps.w[1], w_v, K, dkv, kKT, kFeat) ||
+      !encode_bf16_2d(&maps.a[0], k_in, K, T, kKT, static_cast<uint32_t>(p.box_tok)) ||
+      !encode_bf16_2d(&maps.a[1], v_in, K, T, kKT, static_cast<uint32_t>(p.box_tok)))
+    return KVSHOT_ERR_CUDA;
+  const size_t smem = smem_bytes(p.stages, p.box_tok);
+  if (cudaFuncSetAttribute(kv_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
+      cudaSuccess)
+    return KVSHOT_ERR_CUDA;
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(split);
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  const int pairs = T * d->hkv;  // (token, head) pairs, 4 per CTA
-  cfg.gridDim = dim3(static_cast<unsigned>((pairs + kFinishThreads / 64 - 1) / (kFinishThreads / 64)));
-  cfg.blockDim = dim3(kFinishThreads);
-  cfg.stream = s;
+  cfg.gridDim = dim3(static_cast<unsigned>(split) * static_cast<unsigned>(blocks), static_cast<unsigned>(d->hkv), 2);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = reinterpret_cast<cudaStream_t>(stream);
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kv_project_finish, p) == cudaSuccess ? KVSHOT_OK : KVSHOT_ERR_CUDA;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kv_project_kernel, p, maps) == cudaSuccess ? KVSHOT_OK : KVSHOT_ERR_CUDA;
 }

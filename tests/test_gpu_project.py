@@ -79,6 +79,16 @@ def test_projection_matches_oracle(T, L, hkv, C, paged, P, cap, rope):
     _check(v_pool, v0, vref, rows, "V")
 
 
+# Cluster splits of 8, 4 and 2 CTAs, one and several token blocks (full, one over, one token), uneven shares of the
+# k-tiles (6, 14, 30 over 4 or 8 CTAs) and of the tokens, rings shorter than a CTA's k-tiles.
+@pytest.mark.parametrize("T,L,hkv", [(2, 3, 1), (5, 7, 1), (127, 1, 1), (128, 5, 3), (129, 1, 2), (257, 2, 8), (300, 8, 2),
+                                     (520, 1, 16), (40, 1, 64)])
+def test_projection_splits_and_blocks(T, L, hkv):
+    k_pool, v_pool, k0, v0, kref, vref, rows = _run_case(T, L, hkv, 3, True, 16, 200, True, seed=T + L)
+    _check(k_pool, k0, kref, rows, "K")
+    _check(v_pool, v0, vref, rows, "V")
+
+
 def test_out_of_range_slot_is_reported_and_skipped():
     T, L, hkv, C, cap = 4, 2, 2, 2, 16
     pi = wl.project_inputs(T, L, hkv, device="cuda", seed=3)
