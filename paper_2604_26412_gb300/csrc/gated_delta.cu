@@ -10,17 +10,14 @@
 // Two kernels.  The slab GEMM (kvshot_slab_gemm.cuh, tcgen05 tensor cores)
 // computes the four products of the weight blocks with the token activations,
 // one table entry each:
-//   0: W_g[:, 0:d]   n          2: W_g[:, 2d:3d] o - W_g[:, 2d:3d] n
-//   1: W_g[:, d:2d]  o          3: W_delta o - W_delta n
-// delta is never rounded to bf16: entries 2 and 3 either multiply their
-// weights by n and o stacked along the token axis and subtract the two fp32
-// products (up to 128 tokens per block), or accumulate W o and the
-// negated-weight product W n into one fp32 accumulator (larger blocks); both
-// equal the product with the exact delta up to fp32 rounding.  Each
-// product lands in a workspace slab [4][T][d].  gated_delta_finish, launched
-// behind it with programmatic stream serialization, adds the slabs and
-// applies the gate: h = n + sigmoid(slab0 + slab1 + slab2 + b_g) * slab3,
-// rounded to bf16.
+//   0: W_g[:, 2d:3d] o - W_g[:, 2d:3d] n      2: W_g[:, 0:d]   n
+//   1: W_delta o - W_delta n                  3: W_g[:, d:2d]  o
+// delta is never rounded to bf16: entries 0 and 1 multiply their weights by n
+// and by o and subtract the two fp32 products, which equals the product with the
+// exact delta up to fp32 rounding.  Each product lands in a workspace slab
+// [4][T][d].  gated_delta_finish, launched behind it with programmatic stream
+// serialization, adds the slabs and applies the gate:
+// h = n + sigmoid(slab2 + slab3 + slab0 + b_g) * slab1, rounded to bf16.
 //
 // The step is bound by the weights' bytes (4 d^2 bf16 values, read once:
 // each weight tile is read by the CTAs of every token block at the same time,
@@ -48,19 +45,23 @@ struct FusionParams {
 
 __device__ __forceinline__ float sigmoid(float z) { return 1.f / (1.f + __expf(-z)); }
 
-// h = n + sigmoid(slab0 + slab1 + slab2 + b_g) * slab3, four features per thread.
+// h = n + sigmoid(slab2 + slab3 + slab0 + b_g) * slab1, four features per thread.
 __global__ void __launch_bounds__(kFinishThreads) gated_delta_finish(const __grid_constant__ FusionParams p) {
-  wait_for_prerequisite_grid();
+  // n and b_g are not the slab GEMM's results, and whatever came before it is complete once this kernel can start.
   const size_t td = static_cast<size_t>(p.T) * p.d;
   const size_t e = (static_cast<size_t>(blockIdx.x) * kFinishThreads + threadIdx.x) * 4;
-  if (e >= td) return;
-  const int f = static_cast<int>(e % p.d);
-  const float4 s0 = *reinterpret_cast<const float4*>(p.slab + e);
-  const float4 s1 = *reinterpret_cast<const float4*>(p.slab + td + e);
-  const float4 s2 = *reinterpret_cast<const float4*>(p.slab + 2 * td + e);
-  const float4 u = *reinterpret_cast<const float4*>(p.slab + 3 * td + e);
-  const uint2 nb = *reinterpret_cast<const uint2*>(p.n + e);
-  const uint2 bb = *reinterpret_cast<const uint2*>(p.b_g + f);
+  const bool in = e < td;
+  uint2 nb = make_uint2(0, 0), bb = nb;
+  if (in) {
+    nb = *reinterpret_cast<const uint2*>(p.n + e);
+    bb = *reinterpret_cast<const uint2*>(p.b_g + static_cast<int>(e % p.d));
+  }
+  wait_for_prerequisite_grid();
+  if (!in) return;
+  const float4 s2 = *reinterpret_cast<const float4*>(p.slab + e);
+  const float4 u = *reinterpret_cast<const float4*>(p.slab + td + e);
+  const float4 s0 = *reinterpret_cast<const float4*>(p.slab + 2 * td + e);
+  const float4 s1 = *reinterpret_cast<const float4*>(p.slab + 3 * td + e);
   const float2 n01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&nb.x));
   const float2 n23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&nb.y));
   const float2 b01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bb.x));
@@ -117,17 +118,19 @@ extern "C" kvshot_status kvshot_gated_delta(const kvshot_fusion_desc* d, const v
   gp.T = T;
   gp.d_out = D;
   gp.box_tok = std::min(T, sg::kMaxTok);
-  const int nk = D / sg::kKT;
+  gp.nk = D / sg::kKT;
+  const uint32_t box = static_cast<uint32_t>(sg::mma_n(gp.box_tok) / 2);  // token rows per CTA of a pair
   // weight maps: 0 = W_g, 1 = W_delta; activation maps: 0 = n, 1 = o
-  gp.e[0] = sg::Entry{0, 0, -1, 0, 0, 0, nk};      // W_g[:, 0:d] n
-  gp.e[1] = sg::Entry{0, 1, -1, 0, D, 0, nk};      // W_g[:, d:2d] o
-  gp.e[2] = sg::Entry{0, 0, 1, 0, 2 * D, 0, nk};   // W_g[:, 2d:3d] (o - n)
-  gp.e[3] = sg::Entry{1, 0, 1, 0, 0, 0, nk};       // W_delta (o - n)
+  // The entries with two operands take twice the MMAs of the others at more than 128 tokens, so they come first.
+  gp.e[0] = sg::Entry{0, 0, 1, 2 * D};  // W_g[:, 2d:3d] (o - n)
+  gp.e[1] = sg::Entry{1, 0, 1, 0};      // W_delta (o - n)
+  gp.e[2] = sg::Entry{0, 0, -1, 0};     // W_g[:, 0:d] n
+  gp.e[3] = sg::Entry{0, 1, -1, D};     // W_g[:, d:2d] o
   sg::Maps maps;
   if (!encode_bf16_2d(&maps.w[0], w_g, 3 * static_cast<uint64_t>(D), D, sg::kKT, sg::kFeat) ||
       !encode_bf16_2d(&maps.w[1], w_delta, D, D, sg::kKT, sg::kFeat) ||
-      !encode_bf16_2d(&maps.a[0], n, D, T, sg::kKT, static_cast<uint32_t>(gp.box_tok)) ||
-      !encode_bf16_2d(&maps.a[1], o, D, T, sg::kKT, static_cast<uint32_t>(gp.box_tok)))
+      !encode_bf16_2d(&maps.a[0], n, D, T, sg::kKT, box) ||
+      !encode_bf16_2d(&maps.a[1], o, D, T, sg::kKT, box))
     return KVSHOT_ERR_CUDA;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (sg::launch(gp, maps, 4, s) != cudaSuccess) return KVSHOT_ERR_CUDA;

@@ -59,6 +59,15 @@ def test_fusion_matches_oracle(T, d):
     _compare(_run(fi, T, d), _oracle(fi), f"T={T} d={d}")
 
 
+# A pair of CTAs: odd numbers of 128-feature blocks (the last pair half empty), token counts around the pair's shares of
+# 16 and 32 rows, the stacked form's limit and the second token block, rings that wrap (k-tiles over slots) or not.
+@pytest.mark.parametrize("T,d", [(15, 384), (16, 128), (17, 640), (31, 128), (33, 896), (128, 384), (129, 128), (130, 640),
+                                 (255, 384), (511, 384), (513, 128), (70, 1920)])
+def test_fusion_pair_edges(T, d):
+    fi = wl.fusion_inputs(T, d, device="cuda", seed=T + d)
+    _compare(_run(fi, T, d), _oracle(fi), f"T={T} d={d}")
+
+
 def test_fusion_full_width_hybrid_tree_level():
     # The hybrid-tree workload's widest per-depth step: 16 sequences x 12 draft nodes, d = 4096.
     T, d = 16 * 12, wl.HIDDEN
