@@ -332,7 +332,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
   const uint32_t koff0 = g * 128 + (((2 * q4) ^ g) << 4), koff1 = g * 128 + (((2 * q4 + 1) ^ g) << 4);
   const uint32_t voff0 = 2 * q4 * 128 + ((g ^ (2 * q4)) << 4), voff1 = (2 * q4 + 1) * 128 + ((g ^ (2 * q4 + 1)) << 4);
   // Q^T fragments (f16): k-step 4 kh + s on dims 16 (2 q4 + kh) + 4 s + {0, 1}, {2, 3}.
-  uint2 qreg[CF::kQSmem ? 1 : 8];
+  uint2 qreg[CF::kQSmem ? 1 : 8] = {};
   uint2* qf = sm.qf + rg * (8 * NR * 32) + lane;
   auto q_frag = [&](int kstep, int nr) -> uint2 {
     if constexpr (CF::kQSmem) return qf[(kstep * NR + nr) * 32];
