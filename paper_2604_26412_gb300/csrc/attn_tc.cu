@@ -1541,10 +1541,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     tmem_relinquish();
   }
   tc_fence_before();
-  build_plan(p, sm.len, sm.base, len0);  // block-wide barriers inside
+  build_plan<kTileKeys, kCutsEnd2End>(p, sm.len, sm.base, len0);  // block-wide barriers inside
   tc_fence_after();
   const uint32_t tmem = *sm.tmem_base;
-  const Cursor cu = cursor_begin(p, sm.len, sm.base);
+  const Cursor cu = cursor_begin<kTileKeys, kCutsEnd2End>(p, sm.len, sm.base);
   Pipe pipe{nullptr, nullptr, nullptr, 0, reinterpret_cast<volatile int*>(&sm.misc[0]), nullptr};
   if (warp == kProducerWarp || warp == kProducerVWarp) {
     run_producer_tc<kModePair>(p, maps, sm, pipe, cu, nq_box, warp == kProducerWarp ? 0 : 1);
@@ -1579,7 +1579,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <bool kSpread, bool kF8>
+template <bool kSpread, bool kF8, bool kUnits = false>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ TensorMaps maps, int nq_box) {
   constexpr int NK = kF8 ? kF8NK : kNK, NV = kF8 ? kF8NV : kNV;
@@ -1643,10 +1643,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
   }
   tc_fence_before();
-  build_plan(p, sm.len, sm.base, len0);  // block-wide barriers inside
+  constexpr int kCuts = kUnits ? kCutsUnits : kCutsEnd2End;
+  build_plan<kTileKeys, kCuts>(p, sm.len, sm.base, len0);  // block-wide barriers inside
   tc_fence_after();
   const uint32_t tmem = *sm.tmem_base;
-  const Cursor cu = cursor_begin(p, sm.len, sm.base);
+  const Cursor cu = cursor_begin<kTileKeys, kCuts>(p, sm.len, sm.base);
   Pipe pipe{nullptr, nullptr, nullptr, 0, reinterpret_cast<volatile int*>(&sm.misc[0]), nullptr};
   if (warp == kProducerWarp || warp == kProducerVWarp) {
     if constexpr (kF8) run_producer_f8(p, maps, sm, pipe, cu, nq_box, warp == kProducerWarp ? 0 : 1);
@@ -1718,8 +1719,9 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TensorMaps& maps, int nq_b
   }
   const bool f8 = p.fp8 != 0;
   const size_t smem = smem_bytes(p.C, f8);
-  auto* kernel = f8 ? (spread ? attn_tc_kernel<true, true> : attn_tc_kernel<false, true>)
-                    : (spread ? attn_tc_kernel<true, false> : attn_tc_kernel<false, false>);
+  auto* kernel = p.unit_ctas > 0 ? (f8 ? attn_tc_kernel<true, true, true> : attn_tc_kernel<true, false, true>)
+                 : f8            ? (spread ? attn_tc_kernel<true, true> : attn_tc_kernel<false, true>)
+                                 : (spread ? attn_tc_kernel<true, false> : attn_tc_kernel<false, false>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   return launch_maybe_pdl(kernel, dim3(p.num_ctas), dim3(kThreads), smem, pdl, stream, p, maps, nq_box);

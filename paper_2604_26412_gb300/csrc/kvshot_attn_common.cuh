@@ -269,11 +269,19 @@ __device__ __forceinline__ int clamp_len_of(const AttnParams& p, int L) {
   return L;
 }
 
+// Whether a kernel cuts units by themselves: as the call's plan says, or settled when it is compiled (the tcgen05
+// kernels: even an untaken branch here cost their other calls 0.4 us).
+constexpr int kCutsEither = 0, kCutsEnd2End = 1, kCutsUnits = 2;
+template <int kCuts>
+__device__ __forceinline__ bool unit_cuts(const AttnParams& p) {
+  return kCuts == kCutsEither ? p.unit_ctas > 0 : kCuts == kCutsUnits;
+}
+
 // s_len[c] = clamped L_c; s_base[c] = first global tile of cache c (prefix sum of
 // units x tiles per unit).  Whole block participates.  `len0` may hold
 // seq_lens[threadIdx.x], loaded early by the caller (-1: not loaded).  PK, here and below: keys
 // per prefix tile (draft tiles always hold kTileKeys).
-template <int PK = kTileKeys>
+template <int PK = kTileKeys, int kCuts = kCutsEither>
 __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int* s_base, int len0 = -1) {
   const int HR = p.hkv * p.row_blocks;
   for (int c = threadIdx.x; c < p.C; c += blockDim.x) {
@@ -282,6 +290,7 @@ __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int*
     s_base[c + 1] = ((L + PK - 1) / PK + p.draft_tiles) * HR;
   }
   __syncthreads();
+  if (unit_cuts<kCuts>(p)) return;  // one cache: the cut needs its length alone
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     int carry = 0;
@@ -304,6 +313,21 @@ __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int*
 // Tiles of CTA b: [b * tpc, min(T, (b + 1) * tpc)).
 __device__ __forceinline__ int tiles_per_cta(int total, int ctas) { return (total + ctas - 1) / ctas; }
 
+// One cache with CTAs to spare (p.unit_ctas > 0: the CTAs there are for each unit): every unit is cut by itself into
+// `per` pieces of up to `tpc` tiles, piece i of unit u on CTA u * per + i, so that no CTA takes the end of one unit
+// and the start of the next.  (A second piece costs a CTA an epilogue in mid-stream, ~2 us, and another row of
+// partial results.  Attention and merge, 48 rows, 4096 / 16384 tokens: bf16 15.6 -> 13.1 / 22.2 -> 20.8 us, fp8 on the
+// tcgen05 kernel 23.1 -> 16.1 / 31.4 -> 25.2 us; 4 rows, 16384 tokens 16.0 -> 13.3 us.)
+struct UnitCut {
+  int tpc, per;
+};
+__device__ __forceinline__ UnitCut unit_cut(int unit_ctas, int ut) {
+  UnitCut u;
+  u.tpc = (ut + unit_ctas - 1) / unit_ctas;
+  u.per = (ut + u.tpc - 1) / u.tpc;
+  return u;
+}
+
 struct Cursor {
   int t, t_begin, t_end;  // global tile index and this CTA's range
   int c, hr, lt;          // cache, KV head x row block, tile within the unit
@@ -317,9 +341,19 @@ __device__ __forceinline__ void cursor_load_cache(Cursor& cu, const AttnParams& 
   cu.ut = cu.pt + p.draft_tiles;
 }
 
-template <int PK = kTileKeys>
+template <int PK = kTileKeys, int kCuts = kCutsEither>
 __device__ __forceinline__ Cursor cursor_begin(const AttnParams& p, const int* s_len, const int* s_base) {
   Cursor cu;
+  if (unit_cuts<kCuts>(p)) {
+    cu.c = 0;
+    cursor_load_cache<PK>(cu, p, s_len);
+    const UnitCut u = unit_cut(p.unit_ctas, cu.ut);
+    cu.hr = blockIdx.x / u.per;
+    cu.lt = (blockIdx.x - cu.hr * u.per) * u.tpc;
+    cu.t = cu.t_begin = 0;
+    cu.t_end = cu.hr < p.hkv * p.row_blocks ? min(u.tpc, cu.ut - cu.lt) : 0;
+    return cu;
+  }
   const int total = s_base[p.C];
   const int tpc = tiles_per_cta(total, p.num_ctas);
   cu.t_begin = cu.t = min(total, blockIdx.x * tpc);

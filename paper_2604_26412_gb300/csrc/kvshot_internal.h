@@ -78,6 +78,7 @@ struct AttnParams {
   int prefix_tile;          // keys per prefix tile: TK, or kF8PrefixTile (fp8 mma.sync kernel)
   float qscale;             // softmax scale * log2(e): scores are kept in the log2 domain
   int num_ctas;             // persistent grid size
+  int unit_ctas;            // > 0: one cache, units cut by themselves into up to this many pieces (unit_cut)
   int fp8;                  // target K/V are e4m3 codes (KVSHOT_TARGET_FP8)
   int prefix_grouped;       // prefix tiles are staged in the grouped layout (tensor-memory kernel: draft tiles always;
                             // m16n8k16 kernel: draft tiles too)

@@ -43,24 +43,32 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const __grid_co
   const int h = hr / p.row_blocks, rb = hr - h * p.row_blocks;
   const int rr = rb * p.rows_per_unit + r;
   if (r >= p.rows_per_unit || rr >= p.rows_total) return;
-  // First tile of cache c and the total (the prefix sums of build_plan), 32 caches per round.
-  int cbase = 0, total = 0, ut = 0;
-  for (int c0 = 0; c0 < p.C; c0 += 32) {
-    const int cc = c0 + lane;
-    const int utc = cc < p.C ? (clamp_len(p, cc) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles : 0;
-    int below = cc < c ? utc * HR : 0, all = utc * HR;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      below += __shfl_xor_sync(0xffffffffu, below, o);
-      all += __shfl_xor_sync(0xffffffffu, all, o);
+  int b0, b1;  // the CTAs that held the unit
+  if (p.unit_ctas > 0) {
+    const UnitCut cut = unit_cut(p.unit_ctas, (clamp_len(p, 0) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles);
+    b0 = hr * cut.per;
+    b1 = b0 + cut.per - 1;
+  } else {
+    // First tile of cache c and the total (the prefix sums of build_plan), 32 caches per round.
+    int cbase = 0, total = 0, ut = 0;
+    for (int c0 = 0; c0 < p.C; c0 += 32) {
+      const int cc = c0 + lane;
+      const int utc = cc < p.C ? (clamp_len(p, cc) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles : 0;
+      int below = cc < c ? utc * HR : 0, all = utc * HR;
+  #pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        below += __shfl_xor_sync(0xffffffffu, below, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+      }
+      cbase += below;
+      total += all;
+      if (c - c0 >= 0 && c - c0 < 32) ut = __shfl_sync(0xffffffffu, utc, c - c0);
     }
-    cbase += below;
-    total += all;
-    if (c - c0 >= 0 && c - c0 < 32) ut = __shfl_sync(0xffffffffu, utc, c - c0);
+    const int gs = cbase + hr * ut;
+    const int tpc = tiles_per_cta(total, p.num_ctas);
+    b0 = gs / tpc;
+    b1 = (gs + ut - 1) / tpc;
   }
-  const int gs = cbase + hr * ut;
-  const int tpc = tiles_per_cta(total, p.num_ctas);
-  const int b0 = gs / tpc, b1 = (gs + ut - 1) / tpc;
   if (b0 == b1) return;  // the unit lived in one CTA, which wrote the output itself
   wait_for_prerequisite_grid();
   const int np = b1 - b0 + 1;

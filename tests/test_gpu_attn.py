@@ -123,6 +123,20 @@ def test_one_cache_with_and_without_merge(length, num_ctas):
         gh.compare(out, lse, ref_out, ref_lse, f"L={length} flags={flags} ctas={num_ctas}")
 
 
+# One cache cut unit by unit: pieces per unit that divide its tiles or not, more pieces than tiles, CTAs left over, a
+# bound well above the length, dense rows (cut end to end), several merge batches.
+@pytest.mark.parametrize("num_ctas", [0, 17, 24, 61, 152, 400])
+@pytest.mark.parametrize("length,nq", [(5, 3), (1000, 1), (3001, 3), (3001, 12), (2048, 20)])
+def test_one_cache_cut_into_pieces(length, nq, num_ctas):
+    spec, inp, dk, dv, q, N, Nq = _case((3072,), (8, 12), True, True, 16, 32, 8, nq, seed=nq)
+    inp.seq_lens.fill_(length)
+    hc = gh.HostCache(inp)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for flags in (0, kvshot.KVSHOT_FORCE_MMA, kvshot.KVSHOT_FORCE_TC, kvshot.KVSHOT_FORCE_CC):
+        out, lse = _run(spec, inp, dk, dv, q, N, Nq, flags=flags, num_ctas=num_ctas)
+        gh.compare(out, lse, ref_out, ref_lse, f"L={length} nq={nq} flags={flags} ctas={num_ctas}")
+
+
 def test_scale_parameter():
     spec, inp, dk, dv, q, N, Nq = _case((150,), (2, 2), True, True, 16, 32, 8, 2, seed=5)
     hc = gh.HostCache(inp)

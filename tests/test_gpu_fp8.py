@@ -116,6 +116,17 @@ def test_fp8_stacks_of_more_than_128_rows(nq, hq, hkv):
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 blocks nq={nq} {hq}/{hkv} ctas={num_ctas}")
 
 
+@pytest.mark.parametrize("nq", [1, 4, 12, 20])
+def test_fp8_one_cache_cut_into_pieces(nq):
+    case = ((3001,), (8, 12), True, True, 16, 32, 8, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=300 + nq)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for flags in (0, kvshot.KVSHOT_FORCE_MMA, kvshot.KVSHOT_FORCE_TC):
+        for num_ctas in (0, 8, 24, 61, 152):
+            out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, num_ctas)
+            gh.compare(out, lse, ref_out, ref_lse, f"fp8 one cache nq={nq} flags={flags} ctas={num_ctas}")
+
+
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
     spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(((2000, 900), (4, 4), True, True, 16, 32, 8, 4), seed=21)
     a = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
