@@ -127,6 +127,24 @@ def test_fp8_one_cache_cut_into_pieces(nq):
             gh.compare(out, lse, ref_out, ref_lse, f"fp8 one cache nq={nq} flags={flags} ctas={num_ctas}")
 
 
+# The tcgen05 kernel's spread rows split q into two e4m3 parts scaled row by row: rows of very different magnitude, of
+# zeros, with one large element, and full blocks of 1 to 64 rows, over piece counts above the scale slots (8).
+@pytest.mark.parametrize("nq,hq,hkv", [(1, 8, 8), (1, 32, 8), (5, 32, 8), (7, 16, 8), (16, 32, 8), (2, 64, 2)])
+def test_fp8_split_q_rows(nq, hq, hkv):
+    case = ((200, 63, 129, 0, 65), (8, 12), True, True, 16, hq, hkv, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=400 + nq)
+    g = torch.Generator(device="cuda").manual_seed(nq)
+    scale = 2.0 ** torch.randint(-9, 5, q.shape[:3], generator=g, device="cuda").float()
+    q = (q.float() * scale[..., None]).to(torch.bfloat16)
+    q[0, 0, 0] = 0
+    q[1, :, 1, 7] = 3.0
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    for num_ctas in (0, 1, 7):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, kvshot.KVSHOT_FORCE_TC, num_ctas)
+        # scores up to ~100 here: an error of 2^-17 of the largest element of q moves lse by 2^-17 * 100 < 1e-3
+        gh.compare(out, lse, ref_out, ref_lse, f"fp8 split q nq={nq} {hq}/{hkv} ctas={num_ctas}")
+
+
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
     spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(((2000, 900), (4, 4), True, True, 16, 32, 8, 4), seed=21)
     a = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
