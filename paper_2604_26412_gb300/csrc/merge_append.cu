@@ -16,7 +16,7 @@ using namespace dev;
 
 constexpr int kMergeThreads = 256;
 constexpr int kMergeRows = kMergeThreads / 32;  // rows per CTA, one warp per row
-constexpr int kMergeBatch = 8;                  // pieces whose loads are in flight together (divides 32)
+constexpr int kMergeBatch = 16;                 // pieces whose loads are in flight together (divides 32)
 
 // Workspace slot of the piece computed by CTA b is u + b.  One warp per row
 // of a unit.  Launched behind the attention kernel with programmatic stream
@@ -28,8 +28,10 @@ constexpr int kMergeBatch = 8;                  // pieces whose loads are in fli
 // lse (lane k: piece b0 + k) together with the first kMergeBatch pieces' outputs
 // (lane: 4 dims), and further pieces a batch at a time.  (One piece after another
 // behind the first two, each waiting for its load, the calls of a single cache took
-// 2 us longer: 11 pieces, attention and merge 9.8 -> 7.9 us; 19 pieces 25.9 -> 23.6 us.)
-__global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const __grid_constant__ AttnParams p) {
+// 2 us longer: 11 pieces, attention and merge 9.8 -> 7.9 us in batches of 8, 7.6 of 16;
+// 19 pieces 23.6 us, 22.0, 20.1; batches of 32 19.7 us, but 2 us more for 64 caches,
+// whose rows have 2 or 3 pieces and want more warps.)
+__global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_constant__ AttnParams p) {
   const int blocks_per_unit = (p.rows_per_unit + kMergeRows - 1) / kMergeRows;
   const int u = blockIdx.x / blocks_per_unit;
   const int r = (blockIdx.x - u * blocks_per_unit) * kMergeRows + (threadIdx.x >> 5);
