@@ -285,7 +285,7 @@ kvshot_status make_plan_for(const kvshot_attn_desc* d, bool paged, bool small_bl
   // attn_f8.cu into MMA fragments in registers.  Up to 16 rows the latter streams the codes at
   // 0.84-0.89 of the copy peak (4 rows: 105 us per ragged-chain call, 16 rows: 179 us per multi-layer
   // call, tcgen05 302 and 368 us); its MMAs pad and repeat with the rows, so from 17 rows the tcgen05
-  // kernel is ahead (hybrid tree, 32 and 48 rows: 65 and 66 us per call against 72 and 108 us).  Stacks
+  // kernel is ahead (hybrid tree, 32 and 48 rows: 55 and 56 us per call against 72 and 108 us).  Stacks
   // of more than 128 rows take it in 128-row blocks (the paired kernel has no fp8 form): reading the
   // codes once per block still beats the 64-row blocks of attn_f8.cu (whole hybrid tree, 256 rows:
   // 179 us against 350 us; with the 64-row blocks of the bf16 kernel's fp8 form it was 529 us).
@@ -515,7 +515,7 @@ extern "C" kvshot_status kvshot_draft_attn(const kvshot_attn_desc* d, const void
   // One cache with a CTA per unit, or whose units divide evenly over the CTAs: every CTA takes whole units
   // whatever the length, and nothing is left to merge (tiny chain: one launch of three).
   if (pl.num_ctas == 1 || p.unit_ctas == 1 || (d->num_caches == 1 && pl.units % pl.num_ctas == 0)) return KVSHOT_OK;
-  e = launch_merge(p, s);
+  e = launch_merge(p, sm_count(), s);
   return e == cudaSuccess ? KVSHOT_OK : KVSHOT_ERR_CUDA;
 }
 

@@ -147,7 +147,7 @@ cudaError_t launch_maybe_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, siz
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Actual&&>(args)...);
 }
-cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream);
+cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream);
 cudaError_t launch_append(AppendParams a, cudaStream_t stream);  // with QK-norm when a.q_norm_w is set
 
 // CTAs per SM each kernel variant is built for (its shared-memory ring and

@@ -16,7 +16,6 @@ using namespace dev;
 
 constexpr int kMergeThreads = 256;
 constexpr int kMergeRows = kMergeThreads / 32;  // rows per CTA, one warp per row
-constexpr int kMergeBatch = 16;                 // pieces whose loads are in flight together (divides 32)
 
 // Workspace slot of the piece computed by CTA b is u + b.  One warp per row
 // of a unit.  Launched behind the attention kernel with programmatic stream
@@ -26,12 +25,17 @@ constexpr int kMergeBatch = 16;                 // pieces whose loads are in fli
 // units that lived in one CTA leave at once, and the others only then wait
 // for the attention grid, with one or a few rounds of loads left: every piece's
 // lse (lane k: piece b0 + k) together with the first kMergeBatch pieces' outputs
-// (lane: 4 dims), and further pieces a batch at a time.  (One piece after another
-// behind the first two, each waiting for its load, the calls of a single cache took
-// 2 us longer: 11 pieces, attention and merge 9.8 -> 7.9 us in batches of 8, 7.6 of 16;
-// 19 pieces 23.6 us, 22.0, 20.1; batches of 32 19.7 us, but 2 us more for 64 caches,
-// whose rows have 2 or 3 pieces and want more warps.)
-__global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_constant__ AttnParams p) {
+// (lane: 4 dims; kMergeBatch divides 32), and further pieces a batch at a time.
+// Two forms.  Batches of 16, two CTAs per SM: for the few rows of a small call, each in
+// many pieces.  (One piece after another behind the first two, each waiting for its load,
+// the calls of a single cache took 2 us longer: 11 pieces, attention and merge 9.8 -> 7.9 us
+// in batches of 8, 7.6 of 16; 19 pieces 23.6 us, 22.0, 20.1; of 32 19.7 us.)  Batches of
+// 4 in 40 registers, six CTAs per SM: for calls of more row CTAs than two per SM, whose units are
+// in few pieces and whose waves of CTAs are what costs (16 caches, against batches of 16: 128 rows
+// of 32768 tokens 376 -> 369 us per call, 256 rows of 4096 tokens, nothing split, 75.4 -> 73.9,
+// with an fp8 cache 185 -> 174; batches of 2 the same, of 8 in four CTAs per SM 1 to 2 us more).
+template <int kMergeBatch, int kCtasPerSm>
+__global__ void __launch_bounds__(kMergeThreads, kCtasPerSm) merge_kernel(const __grid_constant__ AttnParams p) {
   const int blocks_per_unit = (p.rows_per_unit + kMergeRows - 1) / kMergeRows;
   const int u = blockIdx.x / blocks_per_unit;
   const int r = (blockIdx.x - u * blocks_per_unit) * kMergeRows + (threadIdx.x >> 5);
@@ -427,7 +431,7 @@ __global__ void __launch_bounds__(kAppendThreads) append_qknorm_kernel(const __g
 
 }  // namespace
 
-cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream) {
+cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream) {
   const int units = p.C * p.hkv * p.row_blocks;
   const int blocks = units * ((p.rows_per_unit + kMergeRows - 1) / kMergeRows);
   cudaLaunchAttribute attr[1];
@@ -440,7 +444,7 @@ cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_kernel, p);
+  return cudaLaunchKernelEx(&cfg, blocks <= 2 * sms ? merge_kernel<16, 2> : merge_kernel<4, 6>, p);
 }
 
 cudaError_t launch_append(AppendParams a, cudaStream_t stream) {

@@ -137,6 +137,19 @@ def test_one_cache_cut_into_pieces(length, nq, num_ctas):
         gh.compare(out, lse, ref_out, ref_lse, f"L={length} nq={nq} flags={flags} ctas={num_ctas}")
 
 
+# The merge's two forms: as many row CTAs as fit two to an SM and one cache more, pieces per row below, at and past a
+# batch, and more than 32.
+@pytest.mark.parametrize("caches", [19, 20])
+@pytest.mark.parametrize("num_ctas", [0, 304, 640, 800, 2900])
+def test_merge_of_many_rows(caches, num_ctas):
+    lens = tuple(2200 if c % 7 == 3 else 100 + 17 * c for c in range(caches))
+    spec, inp, dk, dv, q, N, Nq = _case(lens, (2, 3), True, True, 16, 32, 8, 3, seed=caches)
+    hc = gh.HostCache(inp)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
+    out, lse = _run(spec, inp, dk, dv, q, N, Nq, flags=kvshot.KVSHOT_FORCE_MMA, num_ctas=num_ctas)
+    gh.compare(out, lse, ref_out, ref_lse, f"caches={caches} ctas={num_ctas}")
+
+
 def test_scale_parameter():
     spec, inp, dk, dv, q, N, Nq = _case((150,), (2, 2), True, True, 16, 32, 8, 2, seed=5)
     hc = gh.HostCache(inp)
