@@ -26,19 +26,20 @@ constexpr int kMergeRows = kMergeThreads / 32;  // rows per CTA, one warp per ro
 // for the attention grid, with one or a few rounds of loads left: every piece's
 // lse (lane k: piece b0 + k) together with the first kMergeBatch pieces' outputs
 // (lane: 4 dims; kMergeBatch divides 32), and further pieces a batch at a time.
+// The warps take the rows of all units one after another, whatever a unit's rows are (in CTAs of 8 rows of
+// one unit, padded to the unit's 16, 64 caches of 4 rows took four times the CTAs: step 1562 -> 1532 us).
 // Two forms.  Batches of 16, two CTAs per SM: for the few rows of a small call, each in
 // many pieces.  (One piece after another behind the first two, each waiting for its load,
 // the calls of a single cache took 2 us longer: 11 pieces, attention and merge 9.8 -> 7.9 us
 // in batches of 8, 7.6 of 16; 19 pieces 23.6 us, 22.0, 20.1; of 32 19.7 us.)  Batches of
-// 4 in 40 registers, six CTAs per SM: for calls of more row CTAs than two per SM, whose units are
+// 2 in 40 registers, six CTAs per SM: for calls of more CTAs than two per SM, whose units are
 // in few pieces and whose waves of CTAs are what costs (16 caches, against batches of 16: 128 rows
 // of 32768 tokens 376 -> 369 us per call, 256 rows of 4096 tokens, nothing split, 75.4 -> 73.9,
-// with an fp8 cache 185 -> 174; batches of 2 the same, of 8 in four CTAs per SM 1 to 2 us more).
+// with an fp8 cache 185 -> 174; batches of 4 the same, of 8 in four CTAs per SM 1 to 2 us more).
 template <int kMergeBatch, int kCtasPerSm>
 __global__ void __launch_bounds__(kMergeThreads, kCtasPerSm) merge_kernel(const __grid_constant__ AttnParams p) {
-  const int blocks_per_unit = (p.rows_per_unit + kMergeRows - 1) / kMergeRows;
-  const int u = blockIdx.x / blocks_per_unit;
-  const int r = (blockIdx.x - u * blocks_per_unit) * kMergeRows + (threadIdx.x >> 5);
+  const uint32_t unit_rows = min(p.rows_per_unit, p.rows_total), row = blockIdx.x * kMergeRows + (threadIdx.x >> 5);
+  const int u = row / unit_rows, r = row - u * unit_rows;
   const int lane = threadIdx.x & 31;
   // Rows of unsplit units leave without waiting for the attention grid, so CTA 0 waits for it in any case:
   // a kernel that depends on this grid alone (the next append) then comes after the attention too.
@@ -48,28 +49,29 @@ __global__ void __launch_bounds__(kMergeThreads, kCtasPerSm) merge_kernel(const 
   const int c = u / HR, hr = u - c * HR;
   const int h = hr / p.row_blocks, rb = hr - h * p.row_blocks;
   const int rr = rb * p.rows_per_unit + r;
-  if (r >= p.rows_per_unit || rr >= p.rows_total) return;
+  if (u >= p.C * HR || rr >= p.rows_total) return;
+  const int shift = __ffs(p.prefix_tile) - 1;  // a power of two
+  auto tiles = [&](int len) { return ((len + p.prefix_tile - 1) >> shift) + p.draft_tiles; };
   int b0, b1;  // the CTAs that held the unit
   if (p.unit_ctas > 0) {
-    const UnitCut cut = unit_cut(p.unit_ctas, (clamp_len(p, 0) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles);
+    const UnitCut cut = unit_cut(p.unit_ctas, tiles(clamp_len(p, 0)));
     b0 = hr * cut.per;
     b1 = b0 + cut.per - 1;
   } else {
-    // First tile of cache c and the total (the prefix sums of build_plan), 32 caches per round.
-    int cbase = 0, total = 0, ut = 0;
-    for (int c0 = 0; c0 < p.C; c0 += 32) {
-      const int cc = c0 + lane;
-      const int utc = cc < p.C ? (clamp_len(p, cc) + p.prefix_tile - 1) / p.prefix_tile + p.draft_tiles : 0;
-      int below = cc < c ? utc * HR : 0, all = utc * HR;
-  #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        below += __shfl_xor_sync(0xffffffffu, below, o);
-        all += __shfl_xor_sync(0xffffffffu, all, o);
-      }
-      cbase += below;
-      total += all;
-      if (c - c0 >= 0 && c - c0 < 32) ut = __shfl_sync(0xffffffffu, utc, c - c0);
+    // First tile of cache c and the total (the prefix sums of build_plan): summed per lane, then over the warp once
+    // (a reduction per 32 caches and a division per length made this 8 us of the 89 us of a call of 220 short caches).
+    int below = 0, all = 0;
+    for (int cc = lane; cc < p.C; cc += 32) {
+      const int utc = tiles(clamp_len(p, cc));
+      below += cc < c ? utc : 0;
+      all += utc;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      below += __shfl_xor_sync(0xffffffffu, below, o);
+      all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    const int cbase = below * HR, total = all * HR, ut = tiles(clamp_len(p, c));
     const int gs = cbase + hr * ut;
     const int tpc = tiles_per_cta(total, p.num_ctas);
     b0 = gs / tpc;
@@ -432,8 +434,8 @@ __global__ void __launch_bounds__(kAppendThreads) append_qknorm_kernel(const __g
 }  // namespace
 
 cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream) {
-  const int units = p.C * p.hkv * p.row_blocks;
-  const int blocks = units * ((p.rows_per_unit + kMergeRows - 1) / kMergeRows);
+  const int64_t rows = static_cast<int64_t>(p.C) * p.hkv * p.row_blocks * std::min(p.rows_per_unit, p.rows_total);
+  const int blocks = static_cast<int>((rows + kMergeRows - 1) / kMergeRows);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -444,7 +446,7 @@ cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, blocks <= 2 * sms ? merge_kernel<16, 2> : merge_kernel<4, 6>, p);
+  return cudaLaunchKernelEx(&cfg, blocks <= 2 * sms ? merge_kernel<16, 2> : merge_kernel<2, 6>, p);
 }
 
 cudaError_t launch_append(AppendParams a, cudaStream_t stream) {

@@ -137,9 +137,9 @@ def test_one_cache_cut_into_pieces(length, nq, num_ctas):
         gh.compare(out, lse, ref_out, ref_lse, f"L={length} nq={nq} flags={flags} ctas={num_ctas}")
 
 
-# The merge's two forms: as many row CTAs as fit two to an SM and one cache more, pieces per row below, at and past a
-# batch, and more than 32.
-@pytest.mark.parametrize("caches", [19, 20])
+# The merge's two forms (300 and 312 CTAs of 8 rows, which are 12 to a unit): pieces per row below, at and past a batch,
+# and more than 32.
+@pytest.mark.parametrize("caches", [25, 26])
 @pytest.mark.parametrize("num_ctas", [0, 304, 640, 800, 2900])
 def test_merge_of_many_rows(caches, num_ctas):
     lens = tuple(2200 if c % 7 == 3 else 100 + 17 * c for c in range(caches))
