@@ -1821,7 +1821,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   constexpr int kCuts = kUnits ? kCutsUnits : kCutsEnd2End;
-  build_plan<kTileKeys, kCuts>(p, sm.len, sm.base, len0);  // block-wide barriers inside
+  build_plan<kTileKeys, kCuts, false>(p, sm.len, sm.base, len0);  // block-wide barriers inside
   tc_fence_after();
   const uint32_t tmem = *sm.tmem_base;
   const Cursor cu = cursor_begin<kTileKeys, kCuts>(p, sm.len, sm.base);

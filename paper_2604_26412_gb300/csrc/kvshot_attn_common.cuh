@@ -280,8 +280,11 @@ __device__ __forceinline__ bool unit_cuts(const AttnParams& p) {
 // s_len[c] = clamped L_c; s_base[c] = first global tile of cache c (prefix sum of
 // units x tiles per unit).  Whole block participates.  `len0` may hold
 // seq_lens[threadIdx.x], loaded early by the caller (-1: not loaded).  PK, here and below: keys
-// per prefix tile (draft tiles always hold kTileKeys).
-template <int PK = kTileKeys, int kCuts = kCutsEither>
+// per prefix tile (draft tiles always hold kTileKeys).  kLaneSums: the prefix sum as one scan of the
+// lanes' sums (220 caches of 41..83 tokens, 4 rows: 58.7 -> 53.9 us per call) and not a scan per 32
+// caches, which the tcgen05 kernel of up to 128 rows keeps: it is compiled into 0.4 us less per call with it,
+// with an fp8 cache 1.3.
+template <int PK = kTileKeys, int kCuts = kCutsEither, bool kLaneSums = true>
 __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int* s_base, int len0 = -1) {
   const int HR = p.hkv * p.row_blocks;
   for (int c = threadIdx.x; c < p.C; c += blockDim.x) {
@@ -293,17 +296,35 @@ __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int*
   if (unit_cuts<kCuts>(p)) return;  // one cache: the cut needs its length alone
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
-    int carry = 0;
-    for (int c0 = 0; c0 < p.C; c0 += 32) {
-      const int c = c0 + lane;
-      int v = c < p.C ? s_base[c + 1] : 0;
+    if constexpr (kLaneSums) {
+      // Each lane sums `per` caches, the warp scans the 32 sums once.
+      const int per = (p.C + 31) / 32, c0 = min(p.C, lane * per), c1 = min(p.C, c0 + per);
+      int v = 0;
+      for (int c = c0; c < c1; ++c) v += s_base[c + 1];
+      int scan = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
+        const int t = __shfl_up_sync(0xffffffffu, scan, o);
+        if (lane >= o) scan += t;
       }
-      if (c < p.C) s_base[c + 1] = v + carry;
-      carry += __shfl_sync(0xffffffffu, v, 31);
+      int below = scan - v;
+      for (int c = c0; c < c1; ++c) {
+        below += s_base[c + 1];
+        s_base[c + 1] = below;
+      }
+    } else {
+      int carry = 0;
+      for (int c0 = 0; c0 < p.C; c0 += 32) {
+        const int c = c0 + lane;
+        int v = c < p.C ? s_base[c + 1] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += t;
+        }
+        if (c < p.C) s_base[c + 1] = v + carry;
+        carry += __shfl_sync(0xffffffffu, v, 31);
+      }
     }
     if (lane == 0) s_base[0] = 0;
   }
@@ -534,6 +555,10 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
   int issued = 0;
   int piece = 0;
   bool waited = false;  // griddepcontrol.wait done
+  // Several units per CTA: each is a few tiles, so the first unit's, loaded beside the preceding kernel, are a small
+  // part of the call's and slow that kernel more than they save (220 caches of 41..83 tokens: 55.3 us per level,
+  // 54.5 without; 64 caches of 512..8192 tokens the other way round, 1543 against 1532 us per step).
+  const bool many_units = p.C * p.hkv * p.row_blocks >= 4 * p.num_ctas;
   PageWindow win;
   while (cu.t < cu.t_end) {
     const int h = cu.hr / p.row_blocks;
@@ -541,7 +566,7 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
     const bool draft = cu.lt >= cu.pt;
     const int key0 = (draft ? cu.lt - cu.pt : cu.lt) * kTileKeys;
     const int nkeys = min(kTileKeys, (draft ? p.N : L) - key0);
-    if (draft && !waited) {  // the draft K/V may come from the preceding kernel (KVSHOT_OVERLAP_PREVIOUS)
+    if ((draft || many_units) && !waited) {  // the draft K/V may come from the preceding kernel (KVSHOT_OVERLAP_PREVIOUS)
       wait_for_prerequisite_grid();
       waited = true;
     }
