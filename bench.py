@@ -117,6 +117,7 @@ ATTN_SOURCES = ("attn_cc.cu", "attn_f8.cu", "attn_mma.cu", "attn_tc.cu", "kvshot
 # header, the host planner that sizes its grid, and the merge kernel.  A traffic record names the set
 # its hash covers, so an edit to one kernel leaves the other's record valid.
 MMA_SOURCES = ("attn_mma.cu", "kvshot_api.cu", "kvshot_attn_common.cuh", "kvshot_internal.h", "merge_append.cu")
+F8_SOURCES = ("attn_f8.cu", "kvshot_api.cu", "kvshot_attn_common.cuh", "kvshot_internal.h", "merge_append.cu")
 TC_SOURCES = ("attn_tc.cu", "kvshot_tcgen05.cuh", "kvshot_api.cu", "kvshot_attn_common.cuh", "kvshot_internal.h",
               "merge_append.cu")
 

@@ -77,8 +77,9 @@ typedef enum kvshot_status {
  * draft K/V stay bf16.  Both tensor-core kernels then multiply in f16 (e4m3 -> f16 is exact; q,
  * P and the draft K/V are rounded to f16, which keeps more mantissa than bf16; only magnitudes below
  * 2^-14 lose bits).  Stacks of 17 rows and more run on the tcgen05 kernel (128 rows at a time),
- * which decodes the codes into f16 tiles in shared memory; the others on the m16n8k16 kernel, which
- * decodes them in registers.  KVSHOT_FORCE_TC with more than 128 rows and KVSHOT_FORCE_CC return
+ * which decodes the codes into f16 tiles in shared memory (blocks of 17..64 rows: V's; K's codes are
+ * multiplied as they are by q in two e4m3 parts that hold its bf16 bits, down to 2^-17 of a row's
+ * largest magnitude); the others on the m16n8k16 kernel, which decodes them in registers.  KVSHOT_FORCE_TC with more than 128 rows and KVSHOT_FORCE_CC return
  * KVSHOT_ERR_UNSUPPORTED.  Not in the paper: a cache-compression variant that halves the bytes the
  * kernel reads per target token. */
 #define KVSHOT_TARGET_FP8 0x20u
@@ -209,7 +210,7 @@ kvshot_status kvshot_draft_attn_static(const kvshot_attn_desc* desc, const void*
  *   q_out[c, i, h]              = bf16(rot(q_in[c, i, h]))      for h < hq
  *   draft_k[c, kh, n0 + i]      = bf16(rot(k_in[c, i, kh]))     for kh < hkv
  *   draft_v[c, kh, n0 + i]      = v_in[c, i, kh]                (copied bit for bit)
- * Angles and rotations are computed in fp64 and rounded once to bf16 (nearest even).
+ * The stored values are those of angles and rotations evaluated in fp64 and rounded once to bf16 (nearest even).
  *
  * q_in:  [C, n_new, hq, 128] bf16; k_in, v_in: [C, n_new, hkv, 128] bf16; positions: [C, n_new] int32 >= 0.
  * draft_k/v: [C, hkv, n_max, 128] bf16 (desc->n_max); requires 0 <= n0 and n0 + n_new <= n_max.
@@ -284,8 +285,8 @@ kvshot_status kvshot_gated_delta(const kvshot_fusion_desc* desc, const void* n, 
  * All bf16 pointers 16-byte aligned, int32 pointers 4-byte aligned.  num_layers <= 8, hkv <= 64.
  * Device-side errors (a cache, position or page id out of range) skip that token's store and set
  * KVSHOT_ERR_DEVICE_BOUNDS.  T == 0 is a no-op.
- * Workspace: kvshot_kv_project_workspace_size(desc) bytes (fp32 partial products, 8 L T d_kv bytes), 256-byte aligned,
- * no initialisation needed.
+ * Workspace: kvshot_kv_project_workspace_size(desc) bytes (8 L T d_kv), 256-byte aligned.  It is checked as
+ * before, but not read or written: the partial sums stay on the chip.
  */
 #define KVSHOT_PROJECT_ROPE 0x1u /* re-apply RoPE to the projected keys ("Proj + RoPE fix") */
 
