@@ -134,6 +134,7 @@ constexpr int kAppendThreads = 128;
 constexpr int kAppendCtas = 512;
 constexpr int kAppendSplits = 4;
 constexpr int kAppendGroup = 2;
+constexpr int kNormSplitNodes = 700;
 
 __device__ __noinline__ void sincos_far(double theta, double* sn, double* cs) { sincos(theta, sn, cs); }
 
@@ -451,10 +452,15 @@ cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream) {
 
 cudaError_t launch_append(AppendParams a, cudaStream_t stream) {
   const int nodes = a.C * a.n_new;
-  const int splits = std::max(1, std::min(kAppendSplits, kAppendCtas / nodes));
-  // With QK-norm the angles weigh less than a second wave: 1540 nodes 13.9 us, in CTAs of two nodes 20.5.
-  a.group = a.q_norm_w != nullptr ? 1 : std::max(1, std::min(kAppendGroup, nodes / kAppendCtas));
-  return launch_maybe_pdl(a.q_norm_w != nullptr ? append_qknorm_kernel : append_kernel,
+  const bool norm = a.q_norm_w != nullptr;
+  int splits = std::min(kAppendSplits, kAppendCtas / nodes);
+  // With QK-norm the angles weigh less: two CTAs to a node up to 700 nodes (64 caches of 7 nodes, with the attention
+  // behind it, 56.8 -> 55.0 us; 768 nodes 58.1 against 58.8), and never two nodes to a CTA, whose longer CTAs made a
+  // second wave (1540 nodes 20.5 -> 13.9 us).
+  if (norm) splits = std::max(splits, std::min(2, kNormSplitNodes / nodes * 2));
+  splits = std::max(1, splits);
+  a.group = norm ? 1 : std::max(1, std::min(kAppendGroup, nodes / kAppendCtas));
+  return launch_maybe_pdl(norm ? append_qknorm_kernel : append_kernel,
                           dim3((nodes + a.group - 1) / a.group, splits), dim3(kAppendThreads), 0, true, stream, a);
 }
 
