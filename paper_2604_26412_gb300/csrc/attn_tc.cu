@@ -231,7 +231,9 @@ __device__ __forceinline__ void split_q(uint32_t qbuf, float* qscale, int rows, 
 #pragma unroll
     for (int o = 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
     const uint32_t e = top >> 23;
-    const uint32_t se = e < 8 ? 253u : min(253u, 261u - e);  // the scale's exponent field: 2^7 over the largest's
+    // The scale's exponent field: 2^7 over the largest's.  At most 2^31 (rows of zeros, or below 2^-23): its inverse,
+    // times the smallest score scale of a call (2^-100, kvshot_api.cu), must not vanish, or a masked -inf becomes NaN.
+    const uint32_t se = min(158u, 261u - e);
     const float scale = __uint_as_float(se << 23);
     if (q == 0) qscale[r] = e == 255 ? __uint_as_float(0x7fffffffu) : __uint_as_float((254u - se) << 23);
     uint32_t hi[8], lo[8];

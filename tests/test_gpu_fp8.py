@@ -47,7 +47,7 @@ def _setup(case, seed):
     return spec, inp, dk, dv, q, N, nq, tk8, tv8, hc
 
 
-def _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, num_ctas=0):
+def _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, num_ctas=0, k_exp=wl.FP8_K_EXP, v_exp=wl.FP8_V_EXP, scale=0.0):
     paged = inp.page_table is not None
     out = torch.full(q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
     lse = torch.full(q.shape[:3], float("nan"), dtype=torch.float32, device="cuda")
@@ -57,8 +57,8 @@ def _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, num_ctas=0):
                          page_size=spec.page_size if paged else 0,
                          max_pages_per_seq=inp.page_table.shape[1] if paged else 0,
                          num_pages=inp.num_pages if paged else 0, l_cap=inp.l_cap, tree=spec.tree,
-                         flags=flags | kvshot.KVSHOT_TARGET_FP8, num_ctas=num_ctas, err_flag=err,
-                         k_scale_exp=wl.FP8_K_EXP, v_scale_exp=wl.FP8_V_EXP)
+                         flags=flags | kvshot.KVSHOT_TARGET_FP8, num_ctas=num_ctas, err_flag=err, scale=scale,
+                         k_scale_exp=k_exp, v_scale_exp=v_exp)
     ws = torch.empty(kvshot.workspace_size(d), dtype=torch.uint8, device="cuda")
     d.workspace, d.workspace_bytes = ws.data_ptr(), ws.numel()
     kvshot.draft_attn(d, q, tk8, tv8, inp.page_table, inp.seq_lens, dk, dv, inp.tree_parent[:, :N].contiguous(),
@@ -143,6 +143,21 @@ def test_fp8_split_q_rows(nq, hq, hkv):
         out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, kvshot.KVSHOT_FORCE_TC, num_ctas)
         # scores up to ~100 here: an error of 2^-17 of the largest element of q moves lse by 2^-17 * 100 < 1e-3
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 split q nq={nq} {hq}/{hkv} ctas={num_ctas}")
+
+
+# Rows of zeros and of tiny values where the score scale is smallest: masked keys of a part-filled tile stay masked.
+@pytest.mark.parametrize("k_exp,scale", [(-22, 0.0), (-30, 0.0), (-64, 0.0), (-64, 2.0 ** -90), (-3, 2.0 ** -140)])
+@pytest.mark.parametrize("nq,flags", [(1, 0), (5, 0), (5, kvshot.KVSHOT_FORCE_MMA), (20, 0)])
+def test_fp8_zero_rows_at_small_key_scales(k_exp, scale, nq, flags):
+    case = ((200, 63, 130), (12, 8), True, True, 16, 32, 8, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=500 + nq)
+    hc.tk = of8.dequant_bf16_bits(tk8.cpu().numpy(), k_exp)
+    q[:, 0, 0] = 0
+    q[:, 0, 1] = 2.0 ** -100
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq, scale=scale)
+    for num_ctas in (0, 5):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, num_ctas, k_exp=k_exp, scale=scale)
+        gh.compare(out, lse, ref_out, ref_lse, f"fp8 zero rows nq={nq} k_exp={k_exp} flags={flags} ctas={num_ctas}")
 
 
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
