@@ -118,7 +118,7 @@ struct Smem {
 };
 
 template <class CF>
-__host__ __device__ inline size_t smem_bytes(int C) {
+__host__ __device__ constexpr size_t smem_bytes(int C) {
   size_t off = static_cast<size_t>(CF::kStages) * kStageBytes;
   off += CF::kQBytes + 2 * CF::kStages * sizeof(uint64_t);
   off += sizeof(uint64_t) * kMaxTreeNodes + sizeof(int) * kMaxTreeNodes;
@@ -616,9 +616,16 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
 // 16 caches x 4096 tokens at 16 rows.
 using Cfg8 = Cfg<1, 1, 4, 2, 3>;
 using Cfg16 = Cfg<2, 1, 4, 3, 2>;
-using Cfg32 = Cfg<2, 2, 4, 6, 1>;
+using Cfg32 = Cfg<2, 2, 4, 5, 1>;
 using Cfg48 = Cfg<2, 3, 4, 5, 1>;
 using Cfg64 = Cfg<2, 4, 2, 5, 1>;
+
+// Every plan that kMaxCaches allows fits an SM.
+constexpr size_t kMaxSmem = 227 * 1024;
+static_assert(smem_bytes<Cfg8>(kMaxCaches) <= kMaxSmem && smem_bytes<Cfg16>(kMaxCaches) <= kMaxSmem &&
+                  smem_bytes<Cfg32>(kMaxCaches) <= kMaxSmem && smem_bytes<Cfg48>(kMaxCaches) <= kMaxSmem &&
+                  smem_bytes<Cfg64>(kMaxCaches) <= kMaxSmem,
+              "shared memory at the largest number of caches");
 
 template <class CF>
 cudaError_t launch_cfg(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream) {

@@ -160,6 +160,18 @@ def test_fp8_zero_rows_at_small_key_scales(k_exp, scale, nq, flags):
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 zero rows nq={nq} k_exp={k_exp} flags={flags} ctas={num_ctas}")
 
 
+# The largest number of caches at every row padding of both kernels (G = 5: the m16n8k16 kernel at all of them).
+@pytest.mark.parametrize("nq,hq,hkv", [(1, 5, 1), (2, 5, 1), (4, 5, 1), (6, 5, 1), (8, 5, 1), (12, 5, 1), (13, 5, 1),
+                                       (6, 4, 1), (32, 4, 1), (33, 4, 1)])
+def test_fp8_largest_number_of_caches(nq, hq, hkv):
+    lens = [(37 * c) % 90 for c in range(1024)]
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup((lens, (nq + 2,), True, True, 16, hq, hkv, nq), seed=600 + nq)
+    out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
+    some = [0, 1, 500, 977, 978, 1022, 1023]
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq, caches=some)
+    gh.compare(out[some], lse[some], ref_out, ref_lse, f"fp8 1024 caches nq={nq} {hq}/{hkv}")
+
+
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
     spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(((2000, 900), (4, 4), True, True, 16, 32, 8, 4), seed=21)
     a = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
