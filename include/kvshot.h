@@ -77,9 +77,8 @@ typedef enum kvshot_status {
  * draft K/V stay bf16.  Both tensor-core kernels then multiply in f16 (e4m3 -> f16 is exact; q,
  * P and the draft K/V are rounded to f16, which keeps more mantissa than bf16; only magnitudes below
  * 2^-14 lose bits).  Stacks of 17 rows and more run on the tcgen05 kernel (128 rows at a time),
- * which decodes the codes into f16 tiles in shared memory (blocks of 17..64 rows: V's; K's codes are
- * multiplied as they are by q in two e4m3 parts that hold its bf16 bits, down to 2^-17 of a row's
- * largest magnitude); the others on the m16n8k16 kernel, which decodes them in registers.  KVSHOT_FORCE_TC with more than 128 rows and KVSHOT_FORCE_CC return
+ * which decodes the codes into f16 tiles in shared memory; the others on the m16n8k16 kernel, which
+ * decodes them in registers.  KVSHOT_FORCE_TC with more than 128 rows and KVSHOT_FORCE_CC return
  * KVSHOT_ERR_UNSUPPORTED.  Not in the paper: a cache-compression variant that halves the bytes the
  * kernel reads per target token. */
 #define KVSHOT_TARGET_FP8 0x20u

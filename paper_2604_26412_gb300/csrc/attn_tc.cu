@@ -32,12 +32,14 @@
 // 16-token pages takes 4 boxes per tensor instead of 8.  Ring depths (5 K,
 // 6 V) were measured on GB300: the bytes in flight per SM that the rings
 // allow bound how fast one CTA streams.
-// fp8 target cache (dense and spread rows; the default from 17 rows, in blocks of up to 128): the e4m3 codes of
-// V become f16 V ring tiles: the producer warps land them and the softmax warpgroup between tiles decodes them,
-// three tiles ahead of the tile it takes next.  Spread rows multiply the K codes as they land (kind::f8f6f4) by q
-// split into two e4m3 parts, which hold a bf16's eight bits exactly; dense rows, whose q in both forms would not
-// fit, decode K like V.  The draft tiles (and q for them) are converted to f16 by the producers, and these MMAs
-// and every P.V multiply in f16.
+// fp8 target cache (dense and spread rows; the default from 17 rows, in blocks of up to 128): the
+// producer warps land the e4m3 codes of each tile in a landing slot, and the
+// softmax warpgroup between tiles decodes them into the f16 K and V ring tiles
+// (three tiles ahead of the tile it takes next); q and the draft tiles are
+// converted to f16 by the producers and the MMAs multiply in f16.
+// (K codes multiplied as they land, kind::f8f6f4, by q in two e4m3 parts: no faster, 59.3 us against 59.3 for 48 rows
+// and 16 caches of 4096 tokens, and q's elements below 2^-9 of a row's largest lose bits; in three e5m2 parts, which
+// keep them, 75.7 us.)
 #include <cuda_fp16.h>
 
 #include "kvshot_attn_common.cuh"
@@ -63,30 +65,13 @@ constexpr int kBarSoftmax = 1;             // named barrier among the softmax wa
 constexpr uint32_t kTmemCols = 512;        // S0..S3 [0,256), O0 [256,384), O1 [384,512)
 constexpr uint32_t kTmemO = kNS * kTileKeys;
 constexpr int kMiscInts = 22;
-// fp8 (e4m3) target cache: V (dense rows: K and V) rings of f16 tiles, decoded by the softmax warpgroups from
-// landing slots that the producer warps fill.  Spread rows: the K ring holds the codes.
-constexpr int kCodeBytes = kTileKeys * 128;      // a tile's K (or V) codes
-constexpr int kF8NK = 3;                         // dense rows: K tiles (f16)
-constexpr int kF8DirectNK = 6;                   // spread rows: K tiles (codes)
+// fp8 (e4m3) target cache: rings of f16 tiles, decoded by the softmax warpgroups from landing slots
+// that the producer warps fill (8 KB of K codes and 8 KB of V codes each).
+constexpr int kF8NK = 3;
 constexpr int kF8NV = 4;
-constexpr int kScaleSlots = 8;                   // spread rows: pieces whose rows' q scales are kept (see split_q)
-static_assert(kF8DirectNK % 2 == 0, "a K slot must stay with one producer warp, also across draft tiles");
-// Row mode and cache type -> how the kernel stages K and V.
-template <bool kSpread, bool kF8>
-struct Staging {
-  // K codes go to the MMAs as they are, K out of the decode and its ring (48 rows, 16 caches of 4096 / 16384 tokens:
-  // with skip_tile 61.4 -> 55.6 / 198 -> 175 us per call; skip_tile alone 59.0 / 195 us).
-  static constexpr bool kDirect = kF8 && kSpread;
-  static constexpr int NK = kDirect ? kF8DirectNK : kF8 ? kF8NK : kNK;
-  static constexpr int NV = kF8 ? kF8NV : kNV;
-  static constexpr int kKBytes = kDirect ? kCodeBytes : kKVBytes;              // one K ring slot
-  // The softmax warpgroup done with tile t decodes tile t + kAhead.  Dense rows: 3, so that QK^T of a tile never waits
-  // for the warpgroup that will take its softmax.  Spread rows decode V alone, which P.V of the tile needs: 2, whose V
-  // slot P.V of tile t - 2 has left (with 3 the decode waited for P.V of tile t - 1).
-  static constexpr int kAhead = kDirect ? 2 : 3;
-  static constexpr int kLandBytes = !kF8 ? 0 : kDirect ? kCodeBytes : 2 * kCodeBytes;  // landing slot: (K codes,) V codes
-};
+constexpr int kLandBytes = 2 * kTileKeys * 128;  // one landing slot: a tile's K codes then its V codes
 constexpr int kLandSlots = 4;                    // tile t lands in slot t % kLandSlots, freed when it is decoded
+constexpr int kDecodeAhead = 3;                  // the softmax warpgroup done with tile t decodes tile t + 3
 constexpr int kBarDecode0 = 2;                   // named barriers 2, 3: the 128 threads of warpgroup 0, 1
 static_assert(kLandSlots % 2 == 0, "a landing slot must stay with one producer warp (t and t - kLandSlots)");
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: rescale O when the max grows by > 256x
@@ -183,88 +168,6 @@ __device__ __forceinline__ void bf16_to_f16_inplace(uint32_t buf, int bytes, int
   }
 }
 
-// Spread rows put 16 stacked rows in each 32 rows of the q buffer (two 64-dim halves of 128 rows of 128 bytes), so
-// its rows 16..31 of each 32 are free: the first e4m3 part of q (128 rows of 128 codes, 16 of each 32 used) lies over
-// half 0 from its row 16 on, the second over half 1.
-constexpr uint32_t kQPartHi = 16 * 128;       // byte offset of the first part in the q buffer
-constexpr uint32_t kQPartLo = kQRows * 128;   // of the second after the first
-
-__device__ __forceinline__ uint32_t to_e4m3x2(float lo, float hi) {
-  uint16_t r;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-__device__ __forceinline__ float2 from_e4m3x2(uint32_t codes) {
-  uint32_t h;
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"(static_cast<uint16_t>(codes)));
-  return __half22float2(*reinterpret_cast<__half2*>(&h));
-}
-
-// The landed bf16 q block of a spread unit (`rows` stacked rows) by one warp: to f16 in place, for the draft tiles, and
-// into two e4m3 parts for the codes.  A row is scaled by the power of two that puts its largest magnitude in [128, 256)
-// and split as hi = e4m3(x), lo = e4m3(x - hi): a bf16 has eight significant bits, e4m3 four, and x - hi has at
-// most four after rounding to nearest, so hi + lo is x exactly down to the granule 2^-9 of lo (x of at least 2^-10
-// of the row's largest; below, an error of 2^-10, 2^-17 of the largest).  qscale[row]: the inverse scale; NaN
-// for a row that holds an infinity or a NaN.  Eight rows per step, four lanes each, 32 dims to a lane.
-__device__ __forceinline__ void split_q(uint32_t qbuf, float* qscale, int rows, int lane) {
-  const int q = lane & 3;
-  const int steps = (rows + 7) / 8;
-#pragma unroll 1
-  for (int i = 0; i < steps; ++i) {
-    const int r = 8 * i + (lane >> 2), row = (r >> 4) * 32 + (r & 15);
-    const uint32_t from = qbuf + (q >> 1) * (kQRows * 128) + row * 128;  // 16-byte chunks 4 (q & 1) + j of half q / 2
-    uint4 w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = lds128(from + (((4 * (q & 1) + j) ^ (row & 7)) << 4));
-    float x[32];
-    uint32_t top = 0;  // the largest magnitude's bits (NaN above infinity above every number)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t v[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        x[8 * j + 2 * k] = bf16_lo(v[k]);
-        x[8 * j + 2 * k + 1] = bf16_hi(v[k]);
-        top = max(top, max((v[k] << 16) & 0x7fffffffu, v[k] & 0x7fff0000u));
-      }
-    }
-#pragma unroll
-    for (int o = 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-    const uint32_t e = top >> 23;
-    // The scale's exponent field: 2^7 over the largest's.  At most 2^31 (rows of zeros, or below 2^-23): its inverse,
-    // times the smallest score scale of a call (2^-100, kvshot_api.cu), must not vanish, or a masked -inf becomes NaN.
-    const uint32_t se = min(158u, 261u - e);
-    const float scale = __uint_as_float(se << 23);
-    if (q == 0) qscale[r] = e == 255 ? __uint_as_float(0x7fffffffu) : __uint_as_float((254u - se) << 23);
-    uint32_t hi[8], lo[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      uint32_t h2[2], l2[2];
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        const float a = x[4 * k + 2 * v] * scale, b = x[4 * k + 2 * v + 1] * scale;
-        h2[v] = to_e4m3x2(a, b);
-        const float2 back = from_e4m3x2(h2[v]);
-        l2[v] = to_e4m3x2(a - back.x, b - back.y);
-      }
-      hi[k] = h2[0] | (h2[1] << 16);
-      lo[k] = l2[0] | (l2[1] << 16);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      sts128(from + (((4 * (q & 1) + j) ^ (row & 7)) << 4),
-             make_uint4(pack_f16x2_tc(x[8 * j], x[8 * j + 1]), pack_f16x2_tc(x[8 * j + 2], x[8 * j + 3]),
-                        pack_f16x2_tc(x[8 * j + 4], x[8 * j + 5]), pack_f16x2_tc(x[8 * j + 6], x[8 * j + 7])));
-    const uint32_t part = qbuf + kQPartHi + row * 128;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const uint32_t at = part + (((2 * q + j) ^ (row & 7)) << 4);
-      sts128(at, make_uint4(hi[4 * j], hi[4 * j + 1], hi[4 * j + 2], hi[4 * j + 3]));
-      sts128(at + kQPartLo, make_uint4(lo[4 * j], lo[4 * j + 1], lo[4 * j + 2], lo[4 * j + 3]));
-    }
-  }
-}
-
 // Byte offset of 16-byte chunk `ch` (dims 8ch..8ch+7) of key r in a K or V
 // tile of either layout (128-byte swizzle: chunk index XOR row index mod 8).
 __device__ __forceinline__ uint32_t tile_off_tc(int r, int ch, bool grouped) {
@@ -279,10 +182,7 @@ struct Smem {
   uint8_t* kring;      // kNK x K tile
   uint8_t* vring;      // kNV x V tile
   uint8_t* qbuf;       // one q block
-  uint8_t* land;       // fp8 cache: [kLandSlots] landing slots of e4m3 codes ((K codes, then) V codes)
-  uint8_t* dkbuf;      // fp8 cache, spread rows: [2] a producer warp's draft K tile in f16
-  uint64_t* dkfree;    // fp8 cache, spread rows: [2] QK^T of the draft tile in dkbuf completed
-  float* qscale;       // fp8 cache, spread rows: [kScaleSlots][64] 1 / the power of two that scaled a row of q
+  uint8_t* land;       // fp8 cache: [kLandSlots] landing slots of e4m3 codes (K codes, then V codes)
   uint64_t* kfull;     // [kNK]  TMA -> MMA
   uint64_t* kempty;    // [kNK]  QK^T of the slot's tile completed -> TMA
   uint64_t* vfull;     // [kNV]  TMA -> MMA, softmax
@@ -313,38 +213,35 @@ struct Smem {
   int* lkind;          // fp8 cache: [kLandSlots] 1 when the slot's tile is a draft tile (nothing to decode)
 };
 
-template <class ST>
-__host__ __device__ inline size_t smem_bytes(int C) {
-  size_t off = static_cast<size_t>(ST::NK) * ST::kKBytes + static_cast<size_t>(ST::NV) * kKVBytes + kQBufBytes +
-               kLandSlots * ST::kLandBytes + (ST::kDirect ? 2 * kKVBytes : 0);
-  off += sizeof(uint64_t) * (2 * ST::NK + 2 * ST::NV + 2 + 3 * kNS + 3 + 2 * kLandSlots + 3 + 2);
+__host__ __device__ inline size_t smem_bytes(int C, bool f8) {
+  const int nk = f8 ? kF8NK : kNK, nv = f8 ? kF8NV : kNV;
+  size_t off = static_cast<size_t>(nk + nv) * kKVBytes + kQBufBytes + (f8 ? kLandSlots * kLandBytes : 0);
+  off += sizeof(uint64_t) * (2 * nk + 2 * nv + 2 + 3 * kNS + 3 + 2 * kLandSlots + 3);
   off += sizeof(uint64_t) * kMaxTreeNodes + sizeof(int) * kMaxTreeNodes;
-  off += sizeof(float) * 2 * kQRows + (ST::kDirect ? sizeof(float) * kScaleSlots * kSpreadMaxRows : 0);
+  off += sizeof(float) * 2 * kQRows;
   off += sizeof(uint32_t) * 4 + sizeof(int) * kMiscInts;
   off += sizeof(int) * (2 * C + 1) + sizeof(int) * kLandSlots;
   return off + 1024;
 }
 
-template <class ST>
-__device__ Smem carve(uint8_t* raw, int C) {
+__device__ Smem carve(uint8_t* raw, int C, bool f8) {
+  const int nk = f8 ? kF8NK : kNK, nv = f8 ? kF8NV : kNV;
   Smem s;
   uint8_t* p = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
   s.kring = p;
-  p += ST::NK * ST::kKBytes;
+  p += nk * kKVBytes;
   s.vring = p;
-  p += ST::NV * kKVBytes;
+  p += nv * kKVBytes;
   s.qbuf = p;
   p += kQBufBytes;
   s.land = p;
-  p += kLandSlots * ST::kLandBytes;
-  s.dkbuf = p;
-  if (ST::kDirect) p += 2 * kKVBytes;
+  if (f8) p += kLandSlots * kLandBytes;
   uint64_t* b = reinterpret_cast<uint64_t*>(p);
   s.kfull = b;
-  s.kempty = s.kfull + ST::NK;
-  s.vfull = s.kempty + ST::NK;
-  s.vempty = s.vfull + ST::NV;
-  s.qfull = s.vempty + ST::NV;
+  s.kempty = s.kfull + nk;
+  s.vfull = s.kempty + nk;
+  s.vempty = s.vfull + nv;
+  s.qfull = s.vempty + nv;
   s.qempty = s.qfull + 1;
   s.sfull = s.qempty + 1;
   s.sfree = s.sfull + kNS;
@@ -355,12 +252,10 @@ __device__ Smem carve(uint8_t* raw, int C) {
   s.lfree = s.lfull + kLandSlots;
   s.qland = s.lfree + kLandSlots;
   s.dland = s.qland + 1;
-  s.dkfree = s.dland + 2;
-  s.anc = s.dkfree + 2;
+  s.anc = s.dland + 2;
   s.par = reinterpret_cast<int*>(s.anc + kMaxTreeNodes);
   s.comb = reinterpret_cast<float*>(s.par + kMaxTreeNodes);
-  s.qscale = s.comb + 2 * kQRows;
-  s.tmem_base = reinterpret_cast<uint32_t*>(s.qscale + (ST::kDirect ? kScaleSlots * kSpreadMaxRows : 0));
+  s.tmem_base = reinterpret_cast<uint32_t*>(s.comb + 2 * kQRows);
   s.misc = reinterpret_cast<int*>(s.tmem_base + 4);
   s.len = s.misc + kMiscInts;
   s.base = s.len + C;
@@ -378,13 +273,12 @@ __device__ Smem carve(uint8_t* raw, int C) {
 // S = Q K^T of every tile.  Tile t needs its K tile, its S buffer freed by
 // the completion of P.V of tile t - kNS, and (first tile of a piece) the
 // piece's q block.
-template <bool kSpread, bool kF8>
+template <bool kF8>
 __device__ __forceinline__ void run_mma_qk(const AttnParams& p, const Smem& sm, const Pipe& pipe, uint32_t tmem,
                                            Cursor cu) {
   // fp8 cache: q and the tiles are f16 (e4m3 -> f16 is one conversion per two codes).
   constexpr uint32_t idesc = kF8 ? idesc_f16(128, 64, false) : idesc_bf16(128, 64, false);
-  using ST = Staging<kSpread, kF8>;
-  constexpr int NK = ST::NK;
+  constexpr int NK = kF8 ? kF8NK : kNK;
   int piece = 0;
   for (int t = 0; cu.t < cu.t_end; ++t, cursor_next(cu, p, sm.len)) {
     const TileInfo ti = tile_info(cu, p);
@@ -400,25 +294,7 @@ __device__ __forceinline__ void run_mma_qk(const AttnParams& p, const Smem& sm, 
     sm.misc[2] = t + 1;
     tc_fence_after();
     const uint32_t qbase = smem_addr(sm.qbuf);
-    if constexpr (ST::kDirect) {
-      if (!ti.draft) {
-        // K codes as they landed (64 rows of 128 codes) times the two e4m3 parts of q, 32 dims per MMA.
-        const uint32_t kbase = smem_addr(sm.kring + (t % NK) * kCodeBytes);
-#pragma unroll
-        for (int ks = 0; ks < 2 * (kHeadDim / 32); ++ks) {
-          const uint32_t step = (ks & 3) * 32;
-          tc_mma_f8(tmem + (t % kNS) * kTileKeys,
-                    smem_desc_sw128(qbase + (ks >> 2) * kQPartLo + (kQPartHi + step), 16, 1024),
-                    smem_desc_sw128(kbase + step, 16, 1024), idesc_e4m3(128, 64), ks > 0 ? 1u : 0u);
-        }
-        tc_commit(smem_addr(&sm.sfull[t % kNS]));
-        tc_commit(smem_addr(&sm.kempty[t % NK]));
-        if (ti.last) tc_commit(smem_addr(sm.qempty));
-        continue;
-      }
-    }
-    const uint32_t kbase = smem_addr(ST::kDirect ? sm.dkbuf + (t & 1) * kKVBytes
-                                                 : sm.kring + static_cast<size_t>(t % NK) * kKVBytes);
+    const uint32_t kbase = smem_addr(sm.kring + static_cast<size_t>(t % NK) * kKVBytes);
     // K tile: 8-key groups (the MMA's N direction) kGroupBytes apart and the dims 64..127 half
     // kGroupHalfBytes on (grouped layout), or 1 KB and kHalfBytes (halves layout).
     const bool grouped = ti.draft || p.prefix_grouped;
@@ -431,7 +307,6 @@ __device__ __forceinline__ void run_mma_qk(const AttnParams& p, const Smem& sm, 
     }
     tc_commit(smem_addr(&sm.sfull[t % kNS]));
     tc_commit(smem_addr(&sm.kempty[t % NK]));
-    if (ST::kDirect) tc_commit(smem_addr(&sm.dkfree[t & 1]));
     if (ti.last) tc_commit(smem_addr(sm.qempty));
   }
   tc_commit(smem_addr(&sm.mmadone[0]));
@@ -492,10 +367,7 @@ __device__ __forceinline__ void run_mma_pv(const AttnParams& p, const Smem& sm, 
 // swizzles, so every address is one of four per-lane bases plus a constant.  All eight loads of a
 // lane go out before any conversion or store, so that their latencies overlap (K then V quarters one
 // after the other measured 1% slower on the hybrid tree).
-// kK false: V alone (src: its codes).
-template <bool kK>
-__device__ __forceinline__ void decode_e4m3_quarter(uint32_t src, uint32_t dk, uint32_t dv, int lane, int w) {
-  constexpr int n = kK ? 8 : 4;
+__device__ __forceinline__ void decode_e4m3_quarter_kv(uint32_t src, uint32_t dk, uint32_t dv, int lane, int w) {
   const uint32_t c = lane & 7, r0 = lane >> 3;
   const uint32_t s_even = src + r0 * 128 + ((c ^ r0) << 4);
   const uint32_t s_odd = src + (r0 + 4) * 128 + ((c ^ (r0 + 4)) << 4);
@@ -505,14 +377,14 @@ __device__ __forceinline__ void decode_e4m3_quarter(uint32_t src, uint32_t dk, u
   const uint32_t o0 = dh + (r0 + 4) * 128 + ((((2 * c) & 7) ^ (r0 + 4)) << 4);
   const uint32_t o1 = dh + (r0 + 4) * 128 + ((((2 * c + 1) & 7) ^ (r0 + 4)) << 4);
   const uint32_t k0 = 2 * static_cast<uint32_t>(w);
-  uint4 v[n];
+  uint4 v[8];
 #pragma unroll
-  for (int i = 0; i < n; ++i)
-    v[i] = lds128((i & 1 ? s_odd : s_even) + (k0 + ((i >> 1) & 1)) * 1024 + (i >> 2) * kCodeBytes);
+  for (int i = 0; i < 8; ++i)
+    v[i] = lds128((i & 1 ? s_odd : s_even) + (k0 + ((i >> 1) & 1)) * 1024 + (i >> 2) * (kLandBytes / 2));
 #pragma unroll
-  for (int i = 0; i < n; ++i) {
+  for (int i = 0; i < 8; ++i) {
     const uint32_t k = k0 + ((i >> 1) & 1);
-    const uint32_t dst = kK && i < 4 ? dk : dv;
+    const uint32_t dst = i < 4 ? dk : dv;
     const uint32_t ws[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
     uint32_t o[8];
 #pragma unroll
@@ -564,7 +436,8 @@ __device__ __forceinline__ void rescale_o_tmem(const Smem& sm, const Pipe& pipe,
 
 // Moves the cursor to the next tile if that is a prefix tile of the same piece with another one behind it; a role
 // that takes every second tile steps over it at once.  (The fp8 roles, whose loops bound them: the cursor and a tile's
-// checks cost a warp ~600 cycles, 59.6 -> 55.6 us per hybrid-tree call.  The bf16 ones wait for HBM and gain nothing.)
+// checks cost a warp ~600 cycles, 62.0 -> 59.3 us per call of 48 rows and 16 caches of 4096 tokens.  The bf16 ones wait
+// for HBM and gain nothing.)
 __device__ __forceinline__ bool skip_tile(Cursor& cu) {
   if (cu.lt + 1 >= cu.pt || cu.t + 2 >= cu.t_end) return false;
   ++cu.t;
@@ -575,8 +448,7 @@ __device__ __forceinline__ bool skip_tile(Cursor& cu) {
 template <bool kSpread, bool kF8>
 __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm, const Pipe& pipe, uint32_t tmem,
                                             Cursor cu) {
-  using ST = Staging<kSpread, kF8>;
-  constexpr int NK = ST::NK, NV = ST::NV;
+  constexpr int NK = kF8 ? kF8NK : kNK, NV = kF8 ? kF8NV : kNV;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quarter = warp & 3;                 // TMEM lanes this warp may access
   const int wg = warp >> 2;                     // warpgroup: owns tiles t with t % 2 == wg
@@ -601,16 +473,12 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
   bool valid = false, warp_live = false;
   float m_run = -INFINITY, l_run = 0.f;  // l_run: this thread's columns only (spread)
   int t = 0, anc_seq = -1;
-  // fp8 cache, spread rows: this row's inverse q scale times the cache's key scale, read with the piece's first S
-  // (which implies that its q was split); the slot is written again kScaleSlots pieces later, past the S buffers' lead.
-  int piece = -1;
-  bool row_scaled = false;
-  float code_scale = 1.f;
   // fp8 cache: decodes tile y (its codes landed in slot y % kLandSlots) into its K and V ring slots with
   // this warpgroup's 128 threads, or passes a draft tile's landing through (its producer warp filled
-  // the rings).  Tile y is decoded by warpgroup (y + kAhead) % 2 once it is done with tile y - kAhead
-  // (its own tile; the first kAhead tiles before the loop).  The ring-slot waits are unambiguous: that warpgroup
-  // has seen S of tile y - kAhead, so QK^T of tile y - 2 NK and P.V of tile y - 2 NV had completed.
+  // the rings).  Tile y is decoded by warpgroup (y + 1) % 2 once it is done with tile y - kDecodeAhead
+  // (its own tile; tiles 0..2 before the loop), so QK^T of tile y never waits for the warpgroup that
+  // will take its softmax.  The ring-slot waits are unambiguous: that warpgroup has seen S of tile
+  // y - 3, so QK^T of tile y - 2 NK and P.V of tile y - 2 NV had completed.
   const int ntiles = cu.t_end - cu.t_begin;
   auto decode_landed = [&](int y) {
     const int ls = y % kLandSlots;
@@ -618,13 +486,12 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
     const bool landed = good;
     const bool codes = good && sm.lkind[ls] == 0;
     if (codes) {
-      good = (ST::kDirect || mbar_wait(smem_addr(&sm.kempty[y % NK]), ((y / NK) & 1) ^ 1u, p.err, p.wait_ns)) &&
+      good = mbar_wait(smem_addr(&sm.kempty[y % NK]), ((y / NK) & 1) ^ 1u, p.err, p.wait_ns) &&
              mbar_wait(smem_addr(&sm.vempty[y % NV]), ((y / NV) & 1) ^ 1u, p.err, p.wait_ns);
       if (good) {
-        const uint32_t src = smem_addr(sm.land + static_cast<size_t>(ls) * ST::kLandBytes);
-        const uint32_t dv = smem_addr(sm.vring + static_cast<size_t>(y % NV) * kKVBytes);
-        if constexpr (ST::kDirect) decode_e4m3_quarter<false>(src, 0, dv, lane, quarter);
-        else decode_e4m3_quarter<true>(src, smem_addr(sm.kring + static_cast<size_t>(y % NK) * kKVBytes), dv, lane, quarter);
+        const uint32_t src = smem_addr(sm.land + static_cast<size_t>(ls) * kLandBytes);
+        decode_e4m3_quarter_kv(src, smem_addr(sm.kring + static_cast<size_t>(y % NK) * kKVBytes),
+                               smem_addr(sm.vring + static_cast<size_t>(y % NV) * kKVBytes), lane, quarter);
         fence_proxy_async_smem();  // the MMAs read the tiles through the async proxy
       }
     }
@@ -632,7 +499,7 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
     named_barrier_sync(kBarDecode0 + wg, kSoftmaxThreads / 2);
     if (wtid == 0) {
       if (codes && good) {
-        if (!ST::kDirect) mbar_arrive(smem_addr(&sm.kfull[y % NK]));
+        mbar_arrive(smem_addr(&sm.kfull[y % NK]));
         mbar_arrive(smem_addr(&sm.vfull[y % NV]));
       }
       if (landed) {
@@ -646,7 +513,7 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
   // (KVSHOT_OVERLAP_PREVIOUS); the first S needs q, which comes after that anyway.
   wait_for_prerequisite_grid();
   if constexpr (kF8) {
-    for (int y = (wg + ST::kAhead) & 1; y < min(ST::kAhead, ntiles); y += 2) decode_landed(y);
+    for (int y = 1 - wg; y < min(kDecodeAhead, ntiles); y += 2) decode_landed(y);
   }
   for (; cu.t < cu.t_end; cursor_next(cu, p, sm.len)) {
     const TileInfo ti = tile_info(cu, p);
@@ -664,8 +531,6 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
     if (ti.first) {
       m_run = -INFINITY;
       l_run = 0.f;
-      ++piece;
-      row_scaled = false;
     }
     if (ti.draft && tree) {
       const int seq = cu.c / (p.C / p.B);
@@ -712,15 +577,7 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
         }
         const uint64_t vis = v64 >> col0;  // bit j = column col0 + j
         // fp8 cache: the prefix keys' power-of-two scale is part of the score scale.
-        if constexpr (ST::kDirect) {
-          if (!row_scaled) {
-            code_scale = valid ? sm.qscale[(piece % kScaleSlots) * kSpreadMaxRows + r] * p.k_scale : 1.f;
-            row_scaled = true;
-          }
-        } else {
-          code_scale = p.k_scale;
-        }
-        const float qs = (kF8 && !ti.draft) ? qscale * code_scale : qscale;
+        const float qs = (kF8 && !ti.draft) ? qscale * p.k_scale : qscale;
         float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
         // Spread rows keep the raw scores and fold the scale into the exponent's argument,
         // 2^(s qs - m) = ex2(fma(s, qs, -m)), with the row max taken on the raw scores (qs > 0), in
@@ -809,7 +666,7 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
       tc_fence_before();
       mbar_arrive(smem_addr(&sm.pfull[sbuf]));
       if constexpr (kF8) {
-        if (t + ST::kAhead < ntiles) decode_landed(t + ST::kAhead);
+        if (t + kDecodeAhead < ntiles) decode_landed(t + kDecodeAhead);
       }
     }
     if (ti.last) {
@@ -1144,18 +1001,15 @@ __device__ __forceinline__ TileBoxes tile_boxes_f8(const AttnParams& p, const Cu
 }
 
 // Producer warp `role` with an fp8 target cache; its tiles are t % 2 == role.  A prefix tile's e4m3
-// V codes (dense rows: K and V codes) land in landing slot t % kLandSlots once the decode of tile
-// t - kLandSlots has freed it; the softmax warpgroups decode them into the f16 ring tiles (decode_landed in
-// run_softmax), which keeps the decode (and its shared-memory traffic) off this warp.  Spread rows: the K codes
-// land in their K ring slot, where the MMAs read them.  A draft tile (bf16) is loaded straight into its ring slots
-// (spread rows: its K into this warp's draft buffer) and converted to f16 in place here, and its landing slot is
-// passed through (lkind 1) so that every tile takes one phase of its slots' barriers.  q blocks as in
-// run_producer_tc (role 1), converted to f16 here (spread rows: and split, split_q).
-template <bool kSpread>
+// codes land in landing slot t % kLandSlots once the decode of tile t - kLandSlots has freed it; the
+// softmax warpgroups decode them into the f16 ring tiles (decode_landed in run_softmax), which keeps
+// the decode (and its shared-memory traffic) off this warp, whose box issues and waits then bound
+// nothing.  A draft tile (bf16) is loaded straight into its ring slots and converted to f16 in place
+// here, and its landing slot is passed through (lkind 1) so that every tile takes one phase of its
+// slot's barriers.  q blocks as in run_producer_tc (role 1), converted to f16 here.
 __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const TensorMaps& maps, const Smem& sm,
                                                 const Pipe& pipe, Cursor cu, int nq_box, int role) {
-  using ST = Staging<kSpread, true>;
-  constexpr int NK = ST::NK, NV = ST::NV;
+  constexpr int NK = kF8NK, NV = kF8NV;
   const int lane = threadIdx.x & 31;
   const uint64_t policy = l2_policy_evict_first();
   PageWindow win;
@@ -1190,10 +1044,10 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
         if (ok) {
           const int rb = cu.hr - h * p.row_blocks;
           const uint32_t dst = smem_addr(sm.qbuf);
-          const QBox qb = q_box(p.G, nq_box, kSpread);
+          const QBox qb = q_box(p.G, nq_box, nq_box * p.G <= kSpreadMaxRows);
           const int box_rows = qb.heads * qb.nodes;
           const int rows_q = p.G * nq_box;
-          const int nqb = kSpread ? (rows_q + box_rows - 1) / box_rows : 1;
+          const int nqb = nq_box * p.G <= kSpreadMaxRows ? (rows_q + box_rows - 1) / box_rows : 1;
           mbar_arrive_expect_tx(qbar, 2 * nqb * box_rows * 128);
           for (int k = 0; k < nqb; ++k) {
             const int s0 = k * box_rows;
@@ -1211,10 +1065,7 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
         break;
       }
       ++qblocks;
-      if constexpr (kSpread)
-        split_q(smem_addr(sm.qbuf), sm.qscale + (piece % kScaleSlots) * kSpreadMaxRows, p.G * nq_box, lane);
-      else
-        bf16_to_f16_inplace(smem_addr(sm.qbuf), kQBufBytes, lane);
+      bf16_to_f16_inplace(smem_addr(sm.qbuf), kQBufBytes, lane);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
@@ -1233,13 +1084,9 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
     // The wait is unambiguous because kLandSlots is even: the slot's previous release, the decode of
     // tile t - 2 kLandSlots, was waited by this warp before it landed tile t - kLandSlots.  (With an
     // odd count the slot alternates between the two warps and this wait could pass two phases early.)
-    // Spread rows: so is the K slot, once QK^T of tile t - NK (this warp's too) completed.
-    if (lane < (kSpread ? 2 : 1)) {
-      const uint32_t bar = smem_addr(lane == 0 ? &sm.lfree[ls] : &sm.kempty[t % NK]);
-      const uint32_t par = ((lane == 0 ? t / kLandSlots : t / NK) & 1) ^ 1u;
-      ok = mbar_wait(bar, par, p.err, p.wait_ns) && !*pipe.abort;
-    }
-    ok = __all_sync(0xffffffffu, ok);
+    if (lane == 0)
+      ok = mbar_wait(smem_addr(&sm.lfree[ls]), ((t / kLandSlots) & 1) ^ 1u, p.err, p.wait_ns) && !*pipe.abort;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
     if (!ok) {
       if (lane == 0) *pipe.abort = 1;
       break;
@@ -1250,7 +1097,7 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
       int good = 1;
       // This warp waits for the ring slots only at its draft tiles, so by itself it cannot know that the
       // slots' earlier releases have happened (a wait by parity could then pass two phases early).  Tile
-      // t - 1 being decoded means its decoder had seen S of tile t - 4 at least: QK^T of tile t - 4 and P.V of
+      // t - 1 being decoded means its decoder had seen S of tile t - 4: QK^T of tile t - 4 and P.V of
       // tile t - 8 had completed, which makes the waits below unambiguous.  A growing count, not a
       // barrier phase, so the poll cannot be ambiguous itself.
       if (t >= 1) {
@@ -1265,10 +1112,9 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
           }
         }
       }
-      if (lane < 2 && good && !(kSpread && lane == 0 && drafts == 0)) {
-        // K: its ring slot, or (spread rows) this warp's draft buffer, free once QK^T of its last draft tile completed.
-        const uint32_t bar = smem_addr(lane == 1 ? &sm.vempty[vslot] : kSpread ? &sm.dkfree[role] : &sm.kempty[kslot]);
-        const uint32_t par = lane == 1 ? ((t / NV) & 1) ^ 1u : kSpread ? (drafts - 1) & 1 : ((t / NK) & 1) ^ 1u;
+      if (lane < 2 && good) {
+        const uint32_t bar = lane == 0 ? smem_addr(&sm.kempty[kslot]) : smem_addr(&sm.vempty[vslot]);
+        const uint32_t par = ((t / (lane == 0 ? NK : NV)) & 1) ^ 1u;
         good = mbar_wait(bar, par, p.err, p.wait_ns) && !*pipe.abort;
       }
       if (!__all_sync(0xffffffffu, good)) {
@@ -1281,7 +1127,7 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
         waited = true;
       }
       // bf16 draft K/V land in the ring slots and are converted to f16 there.
-      uint8_t* kd = kSpread ? sm.dkbuf + role * kKVBytes : sm.kring + static_cast<size_t>(kslot) * kKVBytes;
+      uint8_t* kd = sm.kring + static_cast<size_t>(kslot) * kKVBytes;
       uint8_t* vd = sm.vring + static_cast<size_t>(vslot) * kKVBytes;
       const uint32_t dbar = smem_addr(&sm.dland[role]);
       if (lane == 0) mbar_arrive_expect_tx(dbar, 2 * tb.bytes);
@@ -1307,19 +1153,14 @@ __device__ __forceinline__ void run_producer_f8(const AttnParams& p, const Tenso
         mbar_arrive(lbar);
       }
     } else {
-      // The codes: K boxes from lanes 0..15, V boxes from lanes 16..31, rows at 128 bytes in order.  Dense rows land
-      // both in the slot, spread rows K in its ring slot.
-      const uint32_t kbar = kSpread ? smem_addr(&sm.kfull[t % NK]) : lbar;
+      // The codes: K boxes from lanes 0..15, V boxes from lanes 16..31, rows at 128 bytes in order.
       if (lane == 0) {
         sm.lkind[ls] = 0;  // released by the arrive below
-        if (kSpread) mbar_arrive_expect_tx(kbar, tb.bytes);
-        mbar_arrive_expect_tx(lbar, (kSpread ? 1 : 2) * tb.bytes);
-        if (kSpread) sm.misc[8 + role] = t + 1;
+        mbar_arrive_expect_tx(lbar, 2 * tb.bytes);
       }
       __syncwarp();
-      uint8_t* land = sm.land + static_cast<size_t>(ls) * ST::kLandBytes;
-      uint8_t* dst = kSpread ? (kv ? land : sm.kring + static_cast<size_t>(t % NK) * kCodeBytes) : land + kv * kCodeBytes;
-      if (i < tb.nbox) tma_load_2d(smem_addr(dst) + tb.off, kv ? &maps.tv : &maps.tk, 0, tb.y, kv ? lbar : kbar, policy);
+      uint8_t* dst = sm.land + static_cast<size_t>(ls) * kLandBytes + kv * (kLandBytes / 2);
+      if (i < tb.nbox) tma_load_2d(smem_addr(dst) + tb.off, kv ? &maps.tv : &maps.tk, 0, tb.y, lbar, policy);
     }
     ++issued;
     if (lane == 0) sm.misc[12 + role] = issued;
@@ -1758,14 +1599,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
 template <bool kSpread, bool kF8, bool kUnits = false>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ TensorMaps maps, int nq_box) {
-  using ST = Staging<kSpread, kF8>;
-  constexpr int NK = ST::NK, NV = ST::NV;
+  constexpr int NK = kF8 ? kF8NK : kNK, NV = kF8 ? kF8NV : kNV;
   extern __shared__ uint8_t smem_raw[];
   if (threadIdx.x == 0) allow_dependent_launch();  // the merge may be scheduled as CTAs finish
   // The plan's lengths are loaded first, so that their latency overlaps the set-up below
   // (a negative length, invalid anyway, is clamped by the ordinary path).
   const int len0 = static_cast<int>(threadIdx.x) < p.C ? p.seq_lens[threadIdx.x] : -1;
-  const Smem sm = carve<ST>(smem_raw, p.C);
+  const Smem sm = carve(smem_raw, p.C, kF8);
   const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 32 && p.paged) {
     // The page-table line of this CTA's first tile, were every length at its bound (exact
@@ -1803,8 +1643,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(smem_addr(sm.qland), 1);
       mbar_init(smem_addr(&sm.dland[0]), 1);
       mbar_init(smem_addr(&sm.dland[1]), 1);
-      mbar_init(smem_addr(&sm.dkfree[0]), 1);
-      mbar_init(smem_addr(&sm.dkfree[1]), 1);
     }
     mbar_init(smem_addr(sm.ofree), kSoftmaxThreads);
     mbar_init(smem_addr(&sm.mmadone[0]), 1);
@@ -1829,12 +1667,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   const Cursor cu = cursor_begin<kTileKeys, kCuts>(p, sm.len, sm.base);
   Pipe pipe{nullptr, nullptr, nullptr, 0, reinterpret_cast<volatile int*>(&sm.misc[0]), nullptr};
   if (warp == kProducerWarp || warp == kProducerVWarp) {
-    if constexpr (kF8) run_producer_f8<kSpread>(p, maps, sm, pipe, cu, nq_box, warp == kProducerWarp ? 0 : 1);
+    if constexpr (kF8) run_producer_f8(p, maps, sm, pipe, cu, nq_box, warp == kProducerWarp ? 0 : 1);
     else run_producer_tc<kSpread ? kModeSpread : kModeDense>(p, maps, sm, pipe, cu, nq_box, warp == kProducerWarp ? 0 : 1);
   } else if (warp == kMmaWarp || warp == kMmaPvWarp) {
     const int stream = warp == kMmaWarp ? 0 : 1;
     if ((threadIdx.x & 31) == 0 && cu.t < cu.t_end) {
-      if (stream == 0) run_mma_qk<kSpread, kF8>(p, sm, pipe, tmem, cu);
+      if (stream == 0) run_mma_qk<kF8>(p, sm, pipe, tmem, cu);
       else run_mma_pv<kF8>(p, sm, pipe, tmem, cu);
       // Every MMA must have completed before TMEM is released.  Each MMA issued reads shared memory
       // whose loads it already waited for, so it finishes; the wait is retried (bounded) if it runs
@@ -1879,7 +1717,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }  // namespace
 
 cudaError_t attn_tc_occupancy(int C, int* ctas_per_sm) {
-  const size_t smem = smem_bytes<Staging<false, false>>(C);
+  const size_t smem = smem_bytes(C, false);
   cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -1897,8 +1735,7 @@ cudaError_t launch_attn_tc(const AttnParams& p, const TensorMaps& maps, int nq_b
                             nq_box);
   }
   const bool f8 = p.fp8 != 0;
-  const size_t smem = f8 ? (spread ? smem_bytes<Staging<true, true>>(p.C) : smem_bytes<Staging<false, true>>(p.C))
-                         : smem_bytes<Staging<false, false>>(p.C);
+  const size_t smem = smem_bytes(p.C, f8);
   auto* kernel = p.unit_ctas > 0 ? (f8 ? attn_tc_kernel<true, true, true> : attn_tc_kernel<true, false, true>)
                  : f8            ? (spread ? attn_tc_kernel<true, true> : attn_tc_kernel<false, true>)
                                  : (spread ? attn_tc_kernel<true, false> : attn_tc_kernel<false, false>);

@@ -502,8 +502,8 @@ extern "C" kvshot_status kvshot_draft_attn(const kvshot_attn_desc* d, const void
   p.fp8 = fp8 ? 1 : 0;
   p.prefix_grouped = prefix_grouped ? 1 : 0;
   p.wait_ns = d->wait_limit_ns != 0 ? d->wait_limit_ns : static_cast<uint32_t>(2000000000u);
-  // The scale of a prefix score is qscale * k_scale (times a row's own scale of 2^-31 or more in the tcgen05 kernel).  It
-  // must not underflow to 0, which would make the masked scores 0 * -inf: below 2^-100 every score vanishes beside 1.
+  // The scale of a prefix score, qscale * k_scale, must not underflow to 0, which would make the masked scores 0 * -inf:
+  // below 2^-100 every score vanishes beside 1.
   p.k_scale = fp8 ? std::max(std::ldexp(1.f, d->k_scale_exp), std::ldexp(1.f, -100) / p.qscale) : 1.f;
   p.v_scale = fp8 ? std::ldexp(1.f, d->v_scale_exp) : 1.f;
 

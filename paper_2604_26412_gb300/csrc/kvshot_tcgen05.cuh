@@ -34,17 +34,6 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
       : "memory");
 }
 
-// kind::f8f6f4: A and B e4m3 (or e5m2) in shared memory, one byte per element, K = 32 per instruction.
-__device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred acc;\n\t"
-      "setp.ne.b32 acc, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, acc;\n\t}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 // D (+)= A * B with A (M rows = TMEM lanes, K along the columns: two 16-bit
 // elements per 32-bit column, K = 16 per instruction in 8 columns) in tensor
 // memory and B in shared memory.
@@ -198,9 +187,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool b_mn_major) 
   return (1u << 4) | ((b_mn_major ? 1u : 0u) << 16) | (static_cast<uint32_t>(N >> 3) << 17) |
          (static_cast<uint32_t>(M >> 4) << 24);
 }
-
-// The same for kind::f8f6f4 with e4m3 A and B (format 0 there, as f16 is in kind::f16), K-major.
-__host__ __device__ constexpr uint32_t idesc_e4m3(int M, int N) { return idesc_f16(M, N, false); }
 
 }  // namespace
 }  // namespace tc

@@ -127,8 +127,8 @@ def test_fp8_one_cache_cut_into_pieces(nq):
             gh.compare(out, lse, ref_out, ref_lse, f"fp8 one cache nq={nq} flags={flags} ctas={num_ctas}")
 
 
-# The tcgen05 kernel's spread rows split q into two e4m3 parts scaled row by row: rows of very different magnitude, of
-# zeros, with one large element, and full blocks of 1 to 64 rows, over piece counts above the scale slots (8).
+# Rows of very different magnitude, of zeros, with one large element, and full blocks of 1 to 64 rows, in one and in
+# many pieces.
 @pytest.mark.parametrize("nq,hq,hkv", [(1, 8, 8), (1, 32, 8), (5, 32, 8), (7, 16, 8), (16, 32, 8), (2, 64, 2)])
 def test_fp8_split_q_rows(nq, hq, hkv):
     case = ((200, 63, 129, 0, 65), (8, 12), True, True, 16, hq, hkv, nq)
@@ -141,8 +141,30 @@ def test_fp8_split_q_rows(nq, hq, hkv):
     ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq)
     for num_ctas in (0, 1, 7):
         out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, kvshot.KVSHOT_FORCE_TC, num_ctas)
-        # scores up to ~100 here: an error of 2^-17 of the largest element of q moves lse by 2^-17 * 100 < 1e-3
         gh.compare(out, lse, ref_out, ref_lse, f"fp8 split q nq={nq} {hq}/{hkv} ctas={num_ctas}")
+
+
+# One channel of q is 2^drop times the others and meets zero keys: the others alone make the scores (of a few units).
+# lse: the codes are exact, and q where f16 holds it (2^-17 and more; below it errs by up to 2^-25), which leaves the fp32
+# sums of 128 products of up to ~4 and of the exponentials: 128 * 4 * 2^-24 = 3e-5, and 1e-5 for exponent and logarithm.
+@pytest.mark.parametrize("drop", [4, 8, 9, 10, 11, 13, 15])
+@pytest.mark.parametrize("nq", [5, 12, 16])
+def test_fp8_small_elements_of_q_beside_a_dominant_one(drop, nq):
+    case = ((5, 63, 130, 1), (12, 8), True, True, 16, 32, 8, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=700 + nq)
+    q = (q.float() * 2.0 ** -drop * 64).to(torch.bfloat16)
+    q[..., 5] = 64.0
+    tk8[..., 5] = 0
+    dk[..., 5] = 0
+    hc.tk = of8.dequant_bf16_bits(tk8.cpu().numpy(), wl.FP8_K_EXP)
+    scale = 2.0 ** (drop - 6)  # q as drawn gives scores of about 1
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq, scale=scale)
+    inexact = int((q.float().abs() < 2.0 ** -17).sum(-1).max())  # elements of a row, times |k| < 5
+    bound = 4e-5 + inexact * 2.0 ** -25 * 5 * scale
+    for flags in (kvshot.KVSHOT_FORCE_TC, kvshot.KVSHOT_FORCE_MMA):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, flags, 5, scale=scale)
+        gh.compare(out, lse, ref_out, ref_lse, f"fp8 dominant channel drop={drop} nq={nq} flags={flags}")
+        assert np.abs(lse.cpu().numpy() - ref_lse).max() <= bound
 
 
 # Rows of zeros and of tiny values where the score scale is smallest: masked keys of a part-filled tile stay masked.
