@@ -25,7 +25,10 @@
 // one 8x8 transpose (movmatrix) per 8 keys x 8 rows.  All shared-memory loads are
 // free of bank conflicts under the TMA's 128-byte swizzle.
 // e4m3 -> f16 is exact; q, P and the draft K/V are rounded to f16; the cache's
-// power-of-two scales are folded into the score scale (keys) and into P (values).
+// power-of-two scales are folded into the score scale (keys) and, from 2^-4 to 2^8, into P (values).  Times P (up to 1)
+// a larger one would overflow f16 and a smaller one cost P's small values their bits: a form of its own (kWideV) applies
+// those to O where a piece leaves the prefix.  (One form for every scale: 1 cache of 300 tokens, 4 rows, 10.5 -> 10.9 us
+// per call; 64 caches of 512 to 8192 tokens 0.4%.)
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -215,10 +218,10 @@ __device__ __forceinline__ void run_producer_codes(const AttnParams& p, const Te
 
 // Combine the KS key-slice warps of each row group and write the piece: the final bf16 output + lse if
 // the piece is the whole unit, else the normalised fp32 partial + log2-domain lse into slot `slot`.
-// o[mt][nr][2 a + e]: dim 16 g + 2 mt + a of row 8 nr + 2 q4 + e (of the warp's rows).
+// `o_scale`: what o is still to be multiplied by.  o[mt][nr][2 a + e]: dim 16 g + 2 mt + a of row 8 nr + 2 q4 + e (of the warp's rows).
 template <class CF>
 __device__ __forceinline__ void finalize(const AttnParams& p, const Smem& sm, int c, int h, int rb, int slot, bool whole,
-                                         float (&o)[8][CF::kNR][4], const float (&m_run)[CF::kNR][2],
+                                         float o_scale, float (&o)[8][CF::kNR][4], const float (&m_run)[CF::kNR][2],
                                          float (&l_run)[CF::kNR][2]) {
   constexpr int NR = CF::kNR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -255,7 +258,7 @@ __device__ __forceinline__ void finalize(const AttnParams& p, const Smem& sm, in
       }
       M[nr][e] = mx;
       Ls[nr][e] = sum;
-      const float w = (m_run[nr][e] == -INFINITY || mx == -INFINITY) ? 0.f : ex2(m_run[nr][e] - mx);
+      const float w = (m_run[nr][e] == -INFINITY || mx == -INFINITY) ? 0.f : ex2(m_run[nr][e] - mx) * o_scale;
 #pragma unroll
       for (int mt = 0; mt < 8; ++mt) {
         o[mt][nr][e] *= w;
@@ -320,7 +323,7 @@ __device__ __forceinline__ void finalize(const AttnParams& p, const Smem& sm, in
   }
 }
 
-template <class CF>
+template <class CF, bool kWideV>
 __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm, const Pipe& pipe, Cursor cu) {
   constexpr int NR = CF::kNR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -344,6 +347,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
   uint32_t phase = 0;
   int piece_lt0 = 0, anc_seq = -1, consumed = 0;
   int h = 0, rb = 0;
+  bool o_codes = kWideV;  // O is in units of the value codes: this warp has had no draft keys of the piece
 
   for (; cu.t < cu.t_end; cursor_next<kPK>(cu, p, sm.len)) {
     const TileInfo ti = tile_info<kPK>(cu, p);
@@ -378,6 +382,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
         m_run[nr][0] = m_run[nr][1] = -INFINITY;
         l_run[nr][0] = l_run[nr][1] = 0.f;
       }
+      o_codes = kWideV;
       if constexpr (CF::kQSmem) named_barrier_sync(kBarConsumers, CF::kWarps * 32);  // Q^T is shared by the key slices
     }
     if (ti.draft && p.tree) {
@@ -397,8 +402,8 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
     const bool codes = !ti.draft;
     const uint32_t vbase = kbase + (codes ? kCodeBytes : kKVTileBytes);
     const bool full = codes && ti.nkeys == kPK;  // every key of the tile is visible to every row
-    // The key scale is part of the score scale, the value scale part of P (the sum keeps the unscaled P).
-    const float qs = codes ? p.qscale * p.k_scale : p.qscale, vs = codes ? p.v_scale : 1.f;
+    // The key scale is part of the score scale, the value scale part of P (kWideV: of O); the sum keeps the unscaled P.
+    const float qs = codes ? p.qscale * p.k_scale : p.qscale, vs = codes && !kWideV ? p.v_scale : 1.f;
 #pragma unroll 1
     for (int kw = ks * CF::kKW; kw < ks * CF::kKW + CF::kKW; kw += kChunk) {
       if (!live || kw >= ti.nkeys) break;
@@ -473,7 +478,8 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
           mx[nr][e] = fmaxf(fmaxf(s[0][nr][e], s[0][nr][2 + e]), fmaxf(s[1][nr][e], s[1][nr][2 + e])) * qs;
           grow |= mx[nr][e] > m_run[nr][e];
         }
-      if (__any_sync(0xffffffffu, grow)) {
+      const bool leave_codes = kWideV && !codes && o_codes;  // warp-uniform
+      if (__any_sync(0xffffffffu, grow || leave_codes)) {
 #pragma unroll
         for (int nr = 0; nr < NR; ++nr)
 #pragma unroll
@@ -485,13 +491,15 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
             const float alpha = ex2(m_run[nr][e] - (v == -INFINITY ? 0.f : v));
             m_run[nr][e] = v;
             l_run[nr][e] *= alpha;
+            const float o_alpha = leave_codes ? alpha * p.v_scale : alpha;
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
-              o[mt][nr][e] *= alpha;
-              o[mt][nr][2 + e] *= alpha;
+              o[mt][nr][e] *= o_alpha;
+              o[mt][nr][2 + e] *= o_alpha;
             }
           }
       }
+      o_codes &= codes;
       // P^T fragments of the chunk's two 16-key steps.
       uint32_t pb[2][NR][2];
 #pragma unroll
@@ -568,13 +576,13 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
     }
     if (ti.last) {
       const bool whole = piece_lt0 == 0 && cu.lt == cu.ut - 1;
-      finalize<CF>(p, sm, cu.c, h, rb, cu.c * HR + cu.hr + blockIdx.x, whole, o, m_run, l_run);
+      finalize<CF>(p, sm, cu.c, h, rb, cu.c * HR + cu.hr + blockIdx.x, whole, o_codes ? p.v_scale : 1.f, o, m_run, l_run);
     }
   }
   if (threadIdx.x == 0) sm.misc[2] = consumed;
 }
 
-template <class CF>
+template <class CF, bool kWideV>
 __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
     attn_f8_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ TensorMaps maps) {
   extern __shared__ uint8_t smem_raw[];
@@ -602,7 +610,7 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
     // With KVSHOT_OVERLAP_PREVIOUS the kernel may have started before the preceding kernel ended: q is
     // read, and outputs are written, only after it has.
     wait_for_prerequisite_grid();
-    run_consumer<CF>(p, sm, pipe, cu);
+    run_consumer<CF, kWideV>(p, sm, pipe, cu);
   }
   __syncthreads();
   if (threadIdx.x == 0) drain_after_abort(p, pipe, sm.misc[2]);
@@ -630,19 +638,20 @@ static_assert(smem_bytes<Cfg8>(kMaxCaches) <= kMaxSmem && smem_bytes<Cfg16>(kMax
 template <class CF>
 cudaError_t launch_cfg(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream) {
   const size_t smem = smem_bytes<CF>(p.C);
-  cudaError_t e = cudaFuncSetAttribute(attn_f8_kernel<CF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  auto* kernel = p.v_scale < 0x1p-4f || p.v_scale > 0x1p8f ? attn_f8_kernel<CF, true> : attn_f8_kernel<CF, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(attn_f8_kernel<CF>, dim3(p.num_ctas), dim3(CF::kThreads), smem, pdl, stream, p, maps);
+  return launch_maybe_pdl(kernel, dim3(p.num_ctas), dim3(CF::kThreads), smem, pdl, stream, p, maps);
 }
 
+// (Both forms have the same shared memory, and registers capped by the same launch bounds.)
 template <class CF>
 cudaError_t occupancy_cfg(int C, int* ctas) {
   const size_t smem = smem_bytes<CF>(C);
-  cudaError_t e = cudaFuncSetAttribute(attn_f8_kernel<CF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(attn_f8_kernel<CF, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, attn_f8_kernel<CF>, CF::kThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, attn_f8_kernel<CF, false>, CF::kThreads, smem);
 }
 
 }  // namespace

@@ -135,10 +135,10 @@ __device__ __forceinline__ float row_max(const float (&s)[N]) {
   return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
 }
 
-// P = 2^(s qs - m) of N raw scores (qs > 0), packed in pairs into pk (bf16, or f16 times vs), and the
+// P = 2^(s qs - m) of N raw scores (qs > 0), packed in pairs into pk (bf16 or f16), and the
 // sum of the unrounded values.  The scale rides in the exponent's FMA, two lanes per instruction.
 template <int N, bool kF16>
-__device__ __forceinline__ float row_exp(const float (&s)[N], float qs, float m, float vs, uint32_t (&pk)[N / 2]) {
+__device__ __forceinline__ float row_exp(const float (&s)[N], float qs, float m, uint32_t (&pk)[N / 2]) {
   const float2 q2 = make_float2(qs, qs), nm2 = make_float2(-m, -m);
   float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -147,7 +147,7 @@ __device__ __forceinline__ float row_exp(const float (&s)[N], float qs, float m,
     const float2 e = make_float2(ex2(x.x), ex2(x.y));
     if (k & 1) acc1 = add2(acc1, e);
     else acc0 = add2(acc0, e);
-    if constexpr (kF16) pk[k] = pack_f16x2_tc(e.x * vs, e.y * vs);
+    if constexpr (kF16) pk[k] = pack_f16x2_tc(e.x, e.y);
     else pk[k] = pack_bf16x2(e.x, e.y);
   }
   return (acc0.x + acc0.y) + (acc1.x + acc1.y);
@@ -472,6 +472,14 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
   int unit_c = -1, unit_hr = -1, h = 0, rr = 0, nl = 0;
   bool valid = false, warp_live = false;
   float m_run = -INFINITY, l_run = 0.f;  // l_run: this thread's columns only (spread)
+  // fp8 cache: O_wg is in units of the codes (v = code * v_scale) while the piece's tiles are prefix tiles; a rescale
+  // takes it out of them at the warpgroup's first draft tile, or the epilogue where a piece ends before one.  (P of prefix
+  // tiles times v_scale, up to 2^8 * v_scale, leaves f16's range from 2^8 on, and was 1% slower at 4096 tokens.)
+  // Dense rows keep O_wg in the codes from 2^-7 to 2^4, where f16 holds P of the draft tiles divided by v_scale (in its
+  // exponent): 64 caches of 1024 tokens, 256 rows, 525 us against 535; spread rows measured 1.5% slower with it.
+  const bool in_codes = kF8 && !kSpread && p.v_scale >= 0x1p-7f && p.v_scale <= 0x1p4f;
+  const float draft_l = in_codes ? p.v_scale : 1.f, draft_m = in_codes ? __log2f(p.v_scale) : 0.f;
+  int piece_t0 = 0;  // first tile of the piece
   int t = 0, anc_seq = -1;
   // fp8 cache: decodes tile y (its codes landed in slot y % kLandSlots) into its K and V ring slots with
   // this warpgroup's 128 threads, or passes a draft tile's landing through (its producer warp filled
@@ -531,6 +539,7 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
     if (ti.first) {
       m_run = -INFINITY;
       l_run = 0.f;
+      piece_t0 = t;
     }
     if (ti.draft && tree) {
       const int seq = cu.c / (p.C / p.B);
@@ -610,24 +619,26 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
         // faster for them.
         const bool grow = valid && (m_run == -INFINITY ? mx != -INFINITY : mx > m_run + kRescaleThreshold);
         const bool rescale_o = grow && m_run != -INFINITY;
+        const bool leave_codes = kF8 && ti.draft && !in_codes && t - 2 >= piece_t0 && cu.lt - 2 < cu.pt;
         if constexpr (kSpread) {
-          if (__any_sync(0xffffffffu, rescale_o)) {
+          if (__any_sync(0xffffffffu, rescale_o) || leave_codes) {
             const float a = rescale_o ? ex2(m_run - mx) : 1.f;
-            rescale_o_tmem<kSpread>(sm, pipe, p, my_o, t, a);
+            rescale_o_tmem<kSpread>(sm, pipe, p, my_o, t, leave_codes ? a * p.v_scale : a);
             l_run *= a;
           }
         } else {
-          any_rescale = __any_sync(0xffffffffu, rescale_o);
+          any_rescale = __any_sync(0xffffffffu, rescale_o) || leave_codes;
           alpha = rescale_o ? ex2(m_run - mx) : 1.f;
           l_run *= alpha;
+          if (leave_codes) alpha *= p.v_scale;
         }
         if (grow) m_run = mx;
-        const float m_use = m_run == -INFINITY ? 0.f : m_run;
+        float m_use = m_run == -INFINITY ? 0.f : m_run;
+        if (kF8 && !kSpread && ti.draft) m_use += draft_m;
+        const float l_unit = kF8 && !kSpread && ti.draft ? draft_l : 1.f;  // the sum keeps the undivided P
         uint32_t pk[kCols / 2];  // P as bf16 pairs over the S columns just read (rows past the stack: zeros)
-        // fp8 cache: P of prefix tiles carries the values' power-of-two scale; the running sum does not.
-        const float vs = (kF8 && !ti.draft) ? p.v_scale : 1.f;
         if constexpr (kSpread) {
-          l_run += row_exp<kCols, kF8>(pr, qs, m_use, vs, pk);
+          l_run += row_exp<kCols, kF8>(pr, qs, m_use, pk);
         } else {
           float ps4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -635,9 +646,9 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
             const float e0 = ex2(pr[2 * j] - m_use), e1 = ex2(pr[2 * j + 1] - m_use);
             ps4[(2 * j) & 3] += e0;
             ps4[(2 * j + 1) & 3] += e1;
-            pk[j] = kF8 ? pack_f16x2_tc(e0 * vs, e1 * vs) : pack_bf16x2(e0 * vs, e1 * vs);
+            pk[j] = kF8 ? pack_f16x2_tc(e0, e1) : pack_bf16x2(e0, e1);
           }
-          l_run += (ps4[0] + ps4[1]) + (ps4[2] + ps4[3]);
+          l_run += ((ps4[0] + ps4[1]) + (ps4[2] + ps4[3])) * l_unit;
         }
         if constexpr (kSpread) tmem_st16x2_16(trow + sbuf * kTileKeys, pk);
         else tmem_st32(trow + sbuf * kTileKeys, pk);
@@ -698,7 +709,11 @@ __device__ __forceinline__ void run_softmax(const AttnParams& p, const Smem& sm,
         const float L = w0 * l_row + w1 * l1;
         const float inv = L > 0.f ? 1.f / L : 0.f;
         // A warpgroup that owned no tile of this piece left O_w untouched: its weight is 0 and O_w is skipped.
-        const float a0 = w0 * inv, a1 = w1 * inv;
+        float a0 = w0 * inv, a1 = w1 * inv;
+        if constexpr (kF8) {  // O_w in units of the codes: always, or while its last tile, t or t - 1, is a prefix tile
+          if (in_codes || ((t & 1) == 0 ? !ti.draft : cu.lt - 1 < cu.pt)) a0 *= p.v_scale;
+          if (in_codes || ((t & 1) == 1 ? !ti.draft : cu.lt - 1 < cu.pt)) a1 *= p.v_scale;
+        }
         const float lse2 = L > 0.f ? M + __log2f(L) : -INFINITY;
         const bool whole = cu.lt == cu.ut - 1 && (cu.t - cu.t_begin) >= cu.lt;
         const int slot = cu.c * HR + cu.hr + blockIdx.x;
@@ -1424,7 +1439,7 @@ __device__ __forceinline__ void run_softmax_pair(const AttnParams& p, const Smem
       if (grow) m_run = mx;
       const float m_use = m_run == -INFINITY ? 0.f : m_run;
       uint32_t pk[kTileKeys / 2];  // P as bf16 pairs (rows past the stack hold zeros)
-      l_run += row_exp<kTileKeys, false>(pr, qscale, m_use, 1.f, pk);
+      l_run += row_exp<kTileKeys, false>(pr, qscale, m_use, pk);
       tmem_st32(my_s + j * kTileKeys, pk);  // P over the S columns just read
     }
     // Only a rescale of O_wg waits for P.V of the previous tile (sfree of its S buffer, which P.V

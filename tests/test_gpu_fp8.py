@@ -167,6 +167,38 @@ def test_fp8_small_elements_of_q_beside_a_dominant_one(drop, nq):
         assert np.abs(lse.cpu().numpy() - ref_lse).max() <= bound
 
 
+# The whole range of value scales, on pieces that end in the prefix, in the draft and on either side of its first tile.
+# Draft values of magnitude 1 (f16 holds them), and none, which leaves the prefix alone however small its scale; out is
+# compared in units of its largest part.
+@pytest.mark.parametrize("v_exp", [-64, -30, -16, -8, -7, -5, -4, 0, 4, 5, 8, 9, 15, 17, 30, 64])
+@pytest.mark.parametrize("nq,flags", [(1, 0), (4, 0), (12, 0), (32, 0), (12, kvshot.KVSHOT_FORCE_MMA), (40, 0)])
+def test_fp8_value_scales(v_exp, nq, flags):
+    case = ((200, 63, 128, 0, 700), (20, 20), True, True, 16, 32, 8, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=800 + nq)
+    hc.tv = of8.dequant_bf16_bits(tv8.cpu().numpy(), v_exp)
+    unit = 2.0 ** (v_exp - wl.FP8_V_EXP)
+    for dvs, top in ((dv, max(1.0, unit)), (torch.where(dv.isnan(), dv, 0), unit)):
+        ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dvs, N, Nq)
+        for num_ctas in (0, 1, 7, 150):
+            out, lse = _run(spec, inp, tk8, tv8, dk, dvs, q, N, Nq, flags, num_ctas, v_exp=v_exp)
+            gh.compare(out.float() / top, lse, ref_out / top, ref_lse, f"fp8 v_exp={v_exp} nq={nq} ctas={num_ctas}")
+
+
+# A chain of several draft tiles behind the prefix.
+@pytest.mark.parametrize("v_exp", [-20, 20])
+@pytest.mark.parametrize("nq,flags", [(2, 0), (16, 0), (12, kvshot.KVSHOT_FORCE_MMA), (16, kvshot.KVSHOT_FORCE_TC)])
+def test_fp8_value_scale_with_several_draft_tiles(nq, flags, v_exp):
+    case = ((200, 63, 0), tuple([1] * 200), False, True, 16, 16, 8, nq)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=850 + nq)
+    hc.tv = of8.dequant_bf16_bits(tv8.cpu().numpy(), v_exp)
+    draft = 2.0 ** (v_exp // 2)
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv * draft, N, Nq)
+    top = max(draft, 2.0 ** (v_exp - wl.FP8_V_EXP))
+    for num_ctas in (0, 1, 5, 30):
+        out, lse = _run(spec, inp, tk8, tv8, dk, dv * draft, q, N, Nq, flags, num_ctas, v_exp=v_exp)
+        gh.compare(out.float() / top, lse, ref_out / top, ref_lse, f"fp8 chain v_exp={v_exp} nq={nq} ctas={num_ctas}")
+
+
 # Rows of zeros and of tiny values where the score scale is smallest: masked keys of a part-filled tile stay masked.
 @pytest.mark.parametrize("k_exp,scale", [(-22, 0.0), (-30, 0.0), (-64, 0.0), (-64, 2.0 ** -90), (-3, 2.0 ** -140)])
 @pytest.mark.parametrize("nq,flags", [(1, 0), (5, 0), (5, kvshot.KVSHOT_FORCE_MMA), (20, 0)])
