@@ -49,6 +49,11 @@ constexpr int kRingBytes = 102 * 1024;
 constexpr int kMaxStages = 5;
 constexpr int kMaxSplit = 8;                 // CTAs per cluster (the portable limit)
 constexpr int kProjectCtas = 288;            // CTAs of 8-CTA clusters resident at a time
+// Limit on a wait of the pipeline.  (tests/test_gpu_project.py builds a copy whose waits give up at once.)
+#ifndef KVSHOT_PROJECT_WAIT_NS
+#define KVSHOT_PROJECT_WAIT_NS kWaitLimitNs
+#endif
+constexpr uint64_t kPipeLimitNs = KVSHOT_PROJECT_WAIT_NS;
 
 struct ProjectParams {
   const int32_t* token_cache;
@@ -105,6 +110,15 @@ __device__ __forceinline__ float2 cluster_load(uint32_t addr, int rank) {
       : "=f"(v.x), "=f"(v.y)
       : "r"(addr), "r"(rank)
       : "memory");
+  return v;
+}
+
+__device__ __forceinline__ int cluster_load_int(uint32_t addr, int rank) {
+  int v;
+  asm volatile("{\n\t.reg .u32 ra;\n\tmapa.shared::cluster.u32 ra, %1, %2;\n\tld.shared::cluster.s32 %0, [ra];\n\t}"
+               : "=r"(v)
+               : "r"(addr), "r"(rank)
+               : "memory");
   return v;
 }
 
@@ -184,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0 && lane == 0) {
     for (int kt = 0; kt < n; ++kt) {
       const int s = kt % p.stages;
-      if (kt >= p.stages) ok = mbar_wait(smem_addr(&empty[s]), (kt / p.stages - 1) & 1, p.err);
+      if (kt >= p.stages) ok = mbar_wait(smem_addr(&empty[s]), (kt / p.stages - 1) & 1, p.err, kPipeLimitNs);
       if (!ok) break;
       const uint32_t bar = smem_addr(&full[s]), dst = smem_addr(base + s * slot);
       mbar_arrive_expect_tx(bar, kABytes + p.box_tok * kKT * 2);
@@ -205,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t idesc = idesc_bf16(kFeat, N, false);
     for (int kt = 0; kt < n; ++kt) {
       const int s = kt % p.stages;
-      ok = mbar_wait(smem_addr(&full[s]), (kt / p.stages) & 1, p.err);
+      ok = mbar_wait(smem_addr(&full[s]), (kt / p.stages) & 1, p.err, kPipeLimitNs);
       if (!ok) break;
       tc_fence_after();
       const uint32_t a0 = smem_addr(base + s * slot), b0 = a0 + kABytes;
@@ -219,17 +233,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_commit(smem_addr(done));  // every MMA this thread issued has completed
   }
   __syncwarp();
-  mbar_wait(smem_addr(done), 0, p.err);
+  if (!mbar_wait(smem_addr(done), 0, p.err, kPipeLimitNs)) *gave_up = 1;
   tc_fence_after();
-  if (threadIdx.x == 0 && *gave_up)  // let the copies in flight land before their memory is used again
+  // A producer that gives up makes the MMA thread give up, which says so before its commit: after `done` every warp knows
+  // whether all loads were consumed, and leaves the ring alone if not.
+  const bool failed = *gave_up;
+  if (failed && threadIdx.x == 0) {  // let the copies and MMAs in flight end before the CTA does
     for (int kt = max(0, issued - p.stages); kt < issued; ++kt)
       mbar_wait(smem_addr(&full[kt % p.stages]), (kt / p.stages) & 1, p.err);
+    mbar_wait(smem_addr(done), 0, p.err);
+  }
   // Partial sums to shared memory, [token][feature], over the ring (every load has been consumed).
   float* sums = reinterpret_cast<float*>(base);
   const int quarter = warp & 3;  // of the TMEM lanes (features); the two warpgroups take alternate chunks of tokens
   const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
 #pragma unroll 1
-  for (int c = warp >> 2; c * 32 < tokens; c += kThreads / 128) {
+  for (int c = warp >> 2; !failed && c * 32 < tokens; c += kThreads / 128) {
     uint32_t x[32];
     tmem_ld32(trow + c * 32, x);
     tmem_wait_ld();
@@ -239,6 +258,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   cluster_sync();
   if (warp == 1) tmem_dealloc(tmem, cols);
+  // A rank that gave up leaves the cluster's sums incomplete: nothing is stored (the error is recorded already).
+  const int rank_failed = lane < split ? cluster_load_int(smem_addr(tmem_base + 1), lane) : 0;
   Slot next = place;
   for (int t = t0; t < t1; t += kThreads / 32) {
     place = next;
@@ -258,6 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       hi.x += b[r].x;
       hi.y += b[r].y;
     }
+    if (__any_sync(0xffffffffu, rank_failed)) break;
     if (!place.in) {
       if (lane == 0) set_error(p.err, KVSHOT_ERR_DEVICE_BOUNDS);
       continue;

@@ -5,11 +5,17 @@ rounding, so |gpu - oracle| <= 2^-8 |oracle| + 1e-3 per element and relative
 L2 <= 3e-3 over the written rows.  Rows the call does not own must be left
 bit for bit as they were.
 """
+import ctypes
+import glob
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
 from oracle import project as po
+from paper_2604_26412_gb300 import build
 from paper_2604_26412_gb300 import kvshot
 from paper_2604_26412_gb300 import workloads as wl
 
@@ -106,3 +112,39 @@ def test_out_of_range_slot_is_reported_and_skipped():
     written = (k_pool.float().abs().sum(dim=1) > 0).nonzero().flatten().tolist()
     expect = sorted(((0 * hkv + h) * cap + 0) for h in range(hkv)) + sorted(((1 * hkv + h) * cap + 3) for h in range(hkv))
     assert sorted(written) == sorted(expect)
+
+
+def test_a_call_that_times_out_stores_nothing(tmp_path):
+    # A copy of the library whose projection gives up on its first unfinished wait: the call ends, records the timeout
+    # and leaves the cache as it was, and the next call of the ordinary library is correct.
+    obj, lib_path = str(tmp_path / "kv_project.o"), str(tmp_path / "libkvshot_impatient.so")
+    kvshot.load()
+    others = [o for o in glob.glob(os.path.join(build.BUILD, "*.o")) if not o.endswith("kv_project.o")]
+    common = [build.nvcc(), *build.ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", build.INCLUDE]
+    subprocess.run([*common, "-DKVSHOT_PROJECT_WAIT_NS=1", "-c", os.path.join(build.CSRC, "kv_project.cu"), "-o", obj],
+                   check=True)
+    subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-o", lib_path, obj, *others], check=True)
+    impatient = ctypes.CDLL(lib_path).kvshot_kv_project
+    impatient.argtypes, impatient.restype = kvshot.load().kvshot_kv_project.argtypes, ctypes.c_int
+    for T, L, hkv in ((5, 1, 1), (32, 4, 8), (200, 3, 8), (300, 8, 16)):
+        cap = 64 + T
+        pi = wl.project_inputs(T, L, hkv, device="cuda", seed=3)
+        k_pool = torch.randn((hkv * cap, D), device="cuda").to(torch.bfloat16)
+        v_pool = torch.randn((hkv * cap, D), device="cuda").to(torch.bfloat16)
+        k0, v0 = k_pool.clone(), v_pool.clone()
+        err = torch.zeros(1, dtype=torch.int32, device="cuda")
+        d = kvshot.make_project_desc(num_tokens=T, num_layers=L, hkv=hkv, num_caches=1, l_cap=cap, err_flag=err)
+        ws = torch.empty(kvshot.kv_project_workspace_size(d), dtype=torch.uint8, device="cuda")
+        d.workspace, d.workspace_bytes = ws.data_ptr(), ws.numel()
+        tc = torch.zeros(T, dtype=torch.int32, device="cuda")
+        ps = torch.arange(T, dtype=torch.int32, device="cuda")
+        args = [ctypes.byref(d), *(t.data_ptr() for t in (pi.k_in, pi.v_in, pi.w_k, pi.w_v, tc, ps)), None,
+                k_pool.data_ptr(), v_pool.data_ptr(), torch.cuda.current_stream().cuda_stream]
+        for _ in range(2):
+            assert impatient(*args) == kvshot.KVSHOT_OK
+        torch.cuda.synchronize()
+        assert int(err.item()) == kvshot.KVSHOT_ERR_TIMEOUT
+        assert torch.equal(k_pool, k0) and torch.equal(v_pool, v0)
+    k_pool, v_pool, k0, v0, kref, vref, rows = _run_case(33, 4, 8, 4, True, 64, 512, True, seed=5)
+    _check(k_pool, k0, kref, rows, "K")
+    _check(v_pool, v0, vref, rows, "V")
