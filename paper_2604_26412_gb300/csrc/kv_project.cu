@@ -20,11 +20,13 @@
 // tokens, rotates the keys, rounds to bf16 and stores both halves of the head into the cache through the page table.
 // What bounds it: the weights' bytes (one decoding step's few tokens, 2 L_s d_kv^2 bf16 values; an SM ingests
 // ~44 KB/us) and the fixed latencies of launch, load, MMA and exchange, which slot and angle look-ups overlap.
-// Measured, 4 layers of 8 heads, back to back in a graph: 1 token 6.7 us, 32 tokens 7.7, 512 tokens 20.4 us; as a
-// GEMM into fp32 slabs per layer and a second kernel to add them 11.8, 12.5 and 21.5 us.
-// The angle pos * rope_base^(-2j/128) is formed and reduced modulo 2 pi in fp64 (from a host table of the
-// frequencies); sine, cosine and the rotation are fp32 (relative error ~1e-7, far below the bf16 rounding that
-// follows).  fp64 sine and cosine cost this latency-bound kernel ~2 us per call on GB300.
+// Measured, 4 layers of 8 heads, back to back in a graph: 1 token 6.2 us, 32 tokens 7.6, 512 tokens 16.8 us; as a
+// GEMM into fp32 slabs per layer and a second kernel to add them 12.5, 12.9 and 21.8 us.
+// The angle pos * rope_base^(-2j/128) is formed and reduced modulo 2 pi in fixed point: the position times the frequency
+// in turns, a 64-bit fraction from the host, keeps the fraction of a turn in its low 64 bits, of which 32 are turned into
+// radians (2^-30; sine, cosine and the rotation are fp32, relative error ~1e-7, far below the bf16 rounding that follows).
+// An SM executes two fp64 lanes per clock: with the reduction in fp64 two clusters of 128 tokens on one SM took 26 us for
+// it alone (2048 tokens of 1 layer of 8 heads 38.4 us per call, now 32.5).
 #include <algorithm>
 #include <cmath>
 
@@ -69,7 +71,7 @@ struct ProjectParams {
   int stages;   // ring slots of a k-tile of weights and one of tokens
   int paged, page_size, max_pages, num_pages, l_cap;
   int rope;
-  double inv_freq[kHeadDim / 2];  // rope_base^(-2j/128), fp64
+  uint64_t turns[kHeadDim / 2];  // rope_base^(-2j/128) / 2 pi modulo 1, in units of 2^-64
 };
 
 // Maps: weights [d_kv, L d_kv] of K and V, boxes {64, 128}; tokens [T, L d_kv], boxes {64, box_tok}.
@@ -87,7 +89,7 @@ __host__ __device__ inline size_t ring_bytes(int stages, int box_tok) {
   return ring > sums ? ring : sums;
 }
 inline size_t smem_bytes(int stages, int box_tok) {
-  return 1024 + (ring_bytes(stages, box_tok) + 1023) / 1024 * 1024 + 8 * (2 * kMaxStages + 1) + 16;
+  return 1024 + (ring_bytes(stages, box_tok) + 1023) / 1024 * 1024 + 8 * (2 * kMaxStages + 1) + 16 + 12 * kTok;
 }
 
 __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -122,38 +124,35 @@ __device__ __forceinline__ int cluster_load_int(uint32_t addr, int rank) {
   return v;
 }
 
-// Where a token's head goes, and the angles of its pairs (j, j + 64) and (j + 1, j + 65).
-struct Slot {
-  bool in;  // the cache, position and page id are in range
-  size_t row;
-  float2 cs, sn;
-};
-__device__ __forceinline__ Slot find_slot(const ProjectParams& p, int tok, int h, int j, int kv) {
-  Slot s;
+// The cache row of a token's head h, or -1 if its cache, position or page id is out of range.
+__device__ __forceinline__ int64_t find_row(const ProjectParams& p, int tok, int h) {
   const int c = p.token_cache[tok], pos = p.positions[tok];
   const int cap = p.paged ? p.max_pages * p.page_size : p.l_cap;
-  s.in = c >= 0 && c < p.C && pos >= 0 && pos < cap;
-  s.row = 0;
-  if (s.in) {
-    if (p.paged) {
-      const int pid = p.page_table[static_cast<size_t>(c) * p.max_pages + pos / p.page_size];
-      s.in = pid >= 0 && pid < p.num_pages;
-      s.row = (static_cast<size_t>(pid) * p.hkv + h) * p.page_size + pos % p.page_size;
-    } else {
-      s.row = (static_cast<size_t>(c) * p.hkv + h) * p.l_cap + pos;
-    }
-  }
-  s.cs = s.sn = make_float2(0.f, 0.f);
-  if (p.rope && kv == 0) {
-    float r[2];
+  if (c < 0 || c >= p.C || pos < 0 || pos >= cap) return -1;
+  if (!p.paged) return (static_cast<int64_t>(c) * p.hkv + h) * p.l_cap + pos;
+  const int pid = p.page_table[static_cast<size_t>(c) * p.max_pages + pos / p.page_size];
+  if (pid < 0 || pid >= p.num_pages) return -1;
+  return (static_cast<int64_t>(pid) * p.hkv + h) * p.page_size + pos % p.page_size;
+}
+
+// The angles of the pairs (j, j + 64) and (j + 1, j + 65) at a position.
+struct Angles {
+  float2 cs, sn;
+};
+__device__ __forceinline__ Angles angles_at(const ProjectParams& p, int pos, int j) {
+  Angles s;
+  float r[2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const double a = static_cast<double>(pos) * p.inv_freq[j + e];
-      r[e] = static_cast<float>(a - 6.283185307179586 * rint(a * 0.15915494309189535));
-    }
-    sincosf(r[0], &s.sn.x, &s.cs.x);
-    sincosf(r[1], &s.sn.y, &s.cs.y);
+  for (int e = 0; e < 2; ++e) {
+    const uint64_t turn = static_cast<uint64_t>(static_cast<uint32_t>(pos)) * p.turns[j + e];
+    const int32_t x = static_cast<int32_t>((turn + 0x80000000ull) >> 32);  // 2^-32 turns, in [-1/2, 1/2)
+    // x * 2 pi / 2^32 rounded about once: x in two exact halves, the constant in two floats
+    const float hi = static_cast<float>(x & ~0xffff), lo = static_cast<float>(x & 0xffff);
+    constexpr float c = 1.46291807926715968e-9f, c2 = static_cast<float>(1.46291807926715968e-9 - c);
+    r[e] = fmaf(hi, c, fmaf(lo, c, hi * c2));
   }
+  sincosf(r[0], &s.sn.x, &s.cs.x);
+  sincosf(r[1], &s.sn.y, &s.cs.y);
   return s;
 }
 
@@ -170,6 +169,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* done = empty + kMaxStages;
   uint32_t* tmem_base = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* gave_up = reinterpret_cast<volatile int*>(tmem_base + 1);  // a wait timed out
+  int64_t* rows = reinterpret_cast<int64_t*>(tmem_base + 2);               // [kTok] cache row of each token of the share
+  int* pos = reinterpret_cast<int*>(rows + kTok);                          // [kTok] its position
   const int k0 = p.nk * rank / split, n = p.nk * (rank + 1) / split - k0;  // this CTA's k-tiles
   const uint32_t cols = N <= 32 ? 32u : N <= 64 ? 64u : 128u;
   if (threadIdx.x == 0) {
@@ -209,12 +210,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!ok) *gave_up = 1;
   }
   __syncwarp();
-  // This CTA's share of the tokens, a warp per token: lane l has pairs (j, j + 64), j = 2 l and 2 l + 1.  The slot
-  // and the angles of a warp's first token are looked up while the loads are in flight.
+  // This CTA's share of the tokens, a warp per token: lane l has pairs (j, j + 64), j = 2 l and 2 l + 1.  While the loads
+  // are in flight, a thread per token looks up where it goes, and each warp forms its first token's angles.
   const int tokens = min(p.box_tok, p.T - tb * p.box_tok);
-  const int t0 = tokens * rank / split + warp, t1 = tokens * (rank + 1) / split, j = 2 * lane;
-  Slot place{};
-  if (t0 < t1) place = find_slot(p, tb * p.box_tok + t0, h, j, kv);
+  const int s0 = tokens * rank / split, t0 = s0 + warp, t1 = tokens * (rank + 1) / split, j = 2 * lane;
+  const bool rope = p.rope && kv == 0;
+  if (threadIdx.x >= kThreads - kTok) {
+    const int i = threadIdx.x - (kThreads - kTok);
+    if (s0 + i < t1) {
+      const int tok = tb * p.box_tok + s0 + i;
+      rows[i] = find_row(p, tok, h);
+      pos[i] = p.positions[tok];
+    }
+  }
+  Angles ang{};
+  if (rope && t0 < t1) ang = angles_at(p, p.positions[tb * p.box_tok + t0], j);
   if (warp == 1 && lane == 0) {
     const uint32_t idesc = idesc_bf16(kFeat, N, false);
     for (int kt = 0; kt < n; ++kt) {
@@ -260,10 +270,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) tmem_dealloc(tmem, cols);
   // A rank that gave up leaves the cluster's sums incomplete: nothing is stored (the error is recorded already).
   const int rank_failed = lane < split ? cluster_load_int(smem_addr(tmem_base + 1), lane) : 0;
-  Slot next = place;
   for (int t = t0; t < t1; t += kThreads / 32) {
-    place = next;
-    if (t + kThreads / 32 < t1) next = find_slot(p, tb * p.box_tok + t + kThreads / 32, h, j, kv);
+    const int64_t row = rows[t - s0];
     const uint32_t at = smem_addr(sums + t * kFeat + j);
     float2 a[kMaxSplit], b[kMaxSplit];
 #pragma unroll
@@ -271,6 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       a[r] = r < split ? cluster_load(at, r) : make_float2(0.f, 0.f);
       b[r] = r < split ? cluster_load(at + 64 * 4, r) : make_float2(0.f, 0.f);
     }
+    if (rope && t > t0) ang = angles_at(p, pos[t - s0], j);
     float2 lo = a[0], hi = b[0];
 #pragma unroll
     for (int r = 1; r < kMaxSplit; ++r) {
@@ -280,16 +289,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       hi.y += b[r].y;
     }
     if (__any_sync(0xffffffffu, rank_failed)) break;
-    if (!place.in) {
+    if (row < 0) {
       if (lane == 0) set_error(p.err, KVSHOT_ERR_DEVICE_BOUNDS);
       continue;
     }
-    if (p.rope && kv == 0) {
+    if (rope) {
       const float2 x = lo, y = hi;
-      lo = make_float2(x.x * place.cs.x - y.x * place.sn.x, x.y * place.cs.y - y.y * place.sn.y);
-      hi = make_float2(y.x * place.cs.x + x.x * place.sn.x, y.y * place.cs.y + x.y * place.sn.y);
+      lo = make_float2(x.x * ang.cs.x - y.x * ang.sn.x, x.y * ang.cs.y - y.y * ang.sn.y);
+      hi = make_float2(y.x * ang.cs.x + x.x * ang.sn.x, y.y * ang.cs.y + x.y * ang.sn.y);
     }
-    __nv_bfloat16* out = (kv ? p.v_out : p.k_out) + place.row * kHeadDim + j;
+    __nv_bfloat16* out = (kv ? p.v_out : p.k_out) + row * kHeadDim + j;
     *reinterpret_cast<uint32_t*>(out) = pack_bf16x2(lo.x, lo.y);
     *reinterpret_cast<uint32_t*>(out + 64) = pack_bf16x2(hi.x, hi.y);
   }
@@ -353,19 +362,35 @@ extern "C" kvshot_status kvshot_kv_project(const kvshot_project_desc* d, const v
   p.hkv = d->hkv;
   p.C = d->num_caches;
   p.nk = L * dkv / kKT;
-  p.box_tok = std::min(T, kTok);
   p.paged = paged ? 1 : 0;
   p.page_size = paged ? d->page_size : 0;
   p.max_pages = paged ? d->max_pages_per_seq : 0;
   p.num_pages = paged ? d->num_pages : 0;
   p.l_cap = paged ? 0 : d->l_cap;
   p.rope = (d->flags & KVSHOT_PROJECT_ROPE) ? 1 : 0;
-  rope_frequencies(d->rope_base, p.inv_freq);
-  // As many CTAs per cluster as keep the grid within one wave (a k-tile each at least).
-  const int blocks = (T + p.box_tok - 1) / p.box_tok;
-  const int64_t clusters = static_cast<int64_t>(2) * d->hkv * blocks;
-  int split = kMaxSplit;
-  while (split > 1 && (clusters * split > kProjectCtas || split > p.nk)) split /= 2;
+  rope_turns(d->rope_base, p.turns);
+  // As many CTAs per cluster as keep the grid within one wave (a k-tile each at least); blocks of equal size.
+  auto blocks_of = [&](int box) { return (T + box - 1) / box; };
+  auto split_of = [&](int box) {
+    const int64_t clusters = static_cast<int64_t>(2) * d->hkv * blocks_of(box);
+    int split = kMaxSplit;
+    while (split > 1 && (clusters * split > kProjectCtas || split > p.nk)) split /= 2;
+    return split;
+  };
+  // Smaller blocks while a warp has more than one token of a block (its slots and angles are the longest part of a narrow
+  // cache's call), and the blocks, which each read the weights again, find free CTAs for it and few weights.  (With
+  // the angles still in fp64, 128 tokens of 1 layer of 1 head 11.9 -> 4.4 us per call in blocks of 16, of 8 heads 9.0 ->
+  // 8.2 in blocks of 64; beyond 8 k-tiles to a CTA the weights cost more: 512 tokens of 4 layers of 8 heads 19.0 us, in
+  // blocks of 64 23.8.)
+  int box = std::min(T, kTok);
+  while (box > 16 && box > 8 * split_of(box)) {
+    const int half = (box / 2 + 15) / 16 * 16;
+    const int split = split_of(half);
+    if (half >= box || split < std::min(4, p.nk) || (p.nk + split - 1) / split > 8) break;
+    box = half;
+  }
+  const int blocks = blocks_of(box), split = split_of(box);
+  p.box_tok = (T + blocks - 1) / blocks;
   p.split = split;
   const int per_cta = (p.nk + split - 1) / split;
   p.stages = std::min({per_cta, kMaxStages, kRingBytes / slot_bytes(p.box_tok)});

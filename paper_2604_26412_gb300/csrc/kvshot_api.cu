@@ -146,6 +146,30 @@ void rope_frequencies(float rope_base, double* inv_freq) {
   std::copy(table, table + kHeadDim / 2, inv_freq);
 }
 
+void rope_turns(float rope_base, uint64_t* turns) {
+  static thread_local float base = 0.f;
+  static thread_local uint64_t table[kHeadDim / 2];
+  if (base != rope_base) {
+    double inv_freq[kHeadDim / 2];
+    rope_frequencies(rope_base, inv_freq);
+    for (int j = 0; j < kHeadDim / 2; ++j) {
+      // m 2^e / 2 pi with 1 / 2 pi to 2^-128: a product of 192 bits in units of 2^(e - 128), moved to units of 2^-64.
+      int e;
+      const uint64_t m = static_cast<uint64_t>(std::ldexp(std::frexp(inv_freq[j], &e), 53));
+      e -= 53;
+      const unsigned __int128 low = static_cast<unsigned __int128>(m) * 0x7f09d5f47d4d3770ull;
+      const unsigned __int128 high = static_cast<unsigned __int128>(m) * 0x28be60db9391054aull + (low >> 64);
+      const int shift = 64 - e;  // right, of {high, low's 64 bits}
+      if (shift >= 192) table[j] = 0;
+      else if (shift >= 64) table[j] = static_cast<uint64_t>(high >> (shift - 64));
+      else if (shift > 0) table[j] = static_cast<uint64_t>(high << (64 - shift)) | static_cast<uint64_t>(low) >> shift;
+      else table[j] = shift > -64 ? static_cast<uint64_t>(low) << -shift : 0;
+    }
+    base = rope_base;
+  }
+  std::copy(table, table + kHeadDim / 2, turns);
+}
+
 namespace {
 
 // 4-D view {128 dims, hq, Nq, C} of q [C, Nq, hq, 128]; a box is one 64-dim

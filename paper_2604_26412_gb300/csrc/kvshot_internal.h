@@ -121,6 +121,8 @@ bool encode_bf16_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t 
 // inv_freq[j] = rope_base^(-2j/128), j in [0, 64).  Each thread keeps the table of its last rope_base (64 pow calls
 // are ~1.3 us of a call's host time).
 void rope_frequencies(float rope_base, double* inv_freq);
+// turns[j] = rope_base^(-2j/128) / 2 pi modulo 1 in units of 2^-64, from the fp64 frequencies (kept like them).
+void rope_turns(float rope_base, uint64_t* turns);
 
 // Kernel launchers (one per translation unit).  Return cudaSuccess or the launch error.  `pdl`:
 // launch with programmatic stream serialization (KVSHOT_OVERLAP_PREVIOUS).

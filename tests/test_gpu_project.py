@@ -88,11 +88,44 @@ def test_projection_matches_oracle(T, L, hkv, C, paged, P, cap, rope):
 # Cluster splits of 8, 4 and 2 CTAs, one and several token blocks (full, one over, one token), uneven shares of the
 # k-tiles (6, 14, 30 over 4 or 8 CTAs) and of the tokens, rings shorter than a CTA's k-tiles.
 @pytest.mark.parametrize("T,L,hkv", [(2, 3, 1), (5, 7, 1), (127, 1, 1), (128, 5, 3), (129, 1, 2), (257, 2, 8), (300, 8, 2),
-                                     (520, 1, 16), (40, 1, 64)])
+                                     (520, 1, 16), (40, 1, 64),
+                                     # smaller blocks: of 16, 32, 64, equal ones that the tokens do not fill
+                                     (17, 1, 1), (33, 1, 1), (100, 1, 8), (129, 3, 8), (200, 3, 2), (257, 1, 1),
+                                     (515, 1, 2)])
 def test_projection_splits_and_blocks(T, L, hkv):
     k_pool, v_pool, k0, v0, kref, vref, rows = _run_case(T, L, hkv, 3, True, 16, 200, True, seed=T + L)
     _check(k_pool, k0, kref, rows, "K")
     _check(v_pool, v0, vref, rows, "V")
+
+
+def test_angles_over_the_whole_range_of_positions():
+    # Positions up to 2^31 - 1 through a page table whose entries share a few pages; every token has a row of its own.
+    P, hkv, L = 256, 2, 1
+    positions = np.array([0, 1, 77, 4098, 32771, 131076, 10 ** 6 + 6, 10 ** 8 + 5, 2 ** 30 + 9, 2 ** 31 - 1], np.int32)
+    T = len(positions)
+    assert len(set(positions % P)) == T
+    pi = wl.project_inputs(T, L, hkv, device="cuda", seed=9)
+    k_pool = torch.zeros((hkv * P, D), dtype=torch.bfloat16, device="cuda")
+    v_pool = torch.zeros_like(k_pool)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for base in (1.0e6, 1.0e4, 0.5):
+        d = kvshot.make_project_desc(num_tokens=T, num_layers=L, hkv=hkv, num_caches=1, page_size=P,
+                                     max_pages_per_seq=2 ** 31 // P - 1, num_pages=1, rope_base=base, err_flag=err)
+        ws = torch.empty(kvshot.kv_project_workspace_size(d), dtype=torch.uint8, device="cuda")
+        d.workspace, d.workspace_bytes = ws.data_ptr(), ws.numel()
+        pt = torch.zeros((1, 2 ** 31 // P), dtype=torch.int32, device="cuda")
+        tc = torch.zeros(T, dtype=torch.int32, device="cuda")
+        inside = positions < (2 ** 31 // P - 1) * P
+        kvshot.kv_project(d, pi.k_in, pi.v_in, pi.w_k, pi.w_v, tc, torch.from_numpy(positions).cuda(), pt, k_pool, v_pool)
+        torch.cuda.synchronize()
+        assert int(err.item()) == kvshot.KVSHOT_ERR_DEVICE_BOUNDS  # the last one is past the capacity
+        err.zero_()
+        bits = lambda t: wl.bf16_bits(t.cpu())  # noqa: E731
+        kref, _ = po.kv_project(bits(pi.k_in), bits(pi.v_in), bits(pi.w_k), bits(pi.w_v), positions, base, True)
+        got = k_pool.double().cpu().numpy().reshape(hkv, P, D)[:, positions % P].transpose(1, 0, 2)[inside]
+        ref = kref.reshape(T, hkv, D)[inside]
+        # the oracle's fp64 angles are themselves off by up to 2^30 * 2^-53 of a radian, a float's 2^-22 rounding more
+        assert (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-3).all(), base
 
 
 def test_out_of_range_slot_is_reported_and_skipped():
