@@ -624,6 +624,7 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
 // 16 caches x 4096 tokens at 16 rows.
 using Cfg8 = Cfg<1, 1, 4, 2, 3>;
 using Cfg16 = Cfg<2, 1, 4, 3, 2>;
+using Cfg16Many = Cfg<2, 1, 4, 2, 2>;
 using Cfg32 = Cfg<2, 2, 4, 5, 1>;
 using Cfg48 = Cfg<2, 3, 4, 5, 1>;
 using Cfg64 = Cfg<2, 4, 2, 5, 1>;
@@ -634,6 +635,11 @@ static_assert(smem_bytes<Cfg8>(kMaxCaches) <= kMaxSmem && smem_bytes<Cfg16>(kMax
                   smem_bytes<Cfg32>(kMaxCaches) <= kMaxSmem && smem_bytes<Cfg48>(kMaxCaches) <= kMaxSmem &&
                   smem_bytes<Cfg64>(kMaxCaches) <= kMaxSmem,
               "shared memory at the largest number of caches");
+
+// The plan takes 8 bytes of shared memory per cache: past this many, two CTAs of three stages no longer fit an SM.
+constexpr size_t kSmSmem = 228 * 1024, kCtaReserved = 1024;
+constexpr bool many_caches(int C) { return 2 * (smem_bytes<Cfg16>(C) + kCtaReserved) > kSmSmem; }
+static_assert(2 * (smem_bytes<Cfg16Many>(kMaxCaches) + kCtaReserved) <= kSmSmem, "two CTAs at any number of caches");
 
 template <class CF>
 cudaError_t launch_cfg(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream) {
@@ -661,7 +667,7 @@ int attn_f8_rows(int rows) { return rows <= 8 ? 8 : std::min(64, (rows + 15) / 1
 cudaError_t attn_f8_occupancy(int rows_per_unit, int C, int* ctas_per_sm) {
   switch (rows_per_unit) {
     case 8: return occupancy_cfg<Cfg8>(C, ctas_per_sm);
-    case 16: return occupancy_cfg<Cfg16>(C, ctas_per_sm);
+    case 16: return many_caches(C) ? occupancy_cfg<Cfg16Many>(C, ctas_per_sm) : occupancy_cfg<Cfg16>(C, ctas_per_sm);
     case 32: return occupancy_cfg<Cfg32>(C, ctas_per_sm);
     case 48: return occupancy_cfg<Cfg48>(C, ctas_per_sm);
     case 64: return occupancy_cfg<Cfg64>(C, ctas_per_sm);
@@ -672,7 +678,7 @@ cudaError_t attn_f8_occupancy(int rows_per_unit, int C, int* ctas_per_sm) {
 cudaError_t launch_attn_f8(const AttnParams& p, const TensorMaps& maps, bool pdl, cudaStream_t stream) {
   switch (p.rows_per_unit) {
     case 8: return launch_cfg<Cfg8>(p, maps, pdl, stream);
-    case 16: return launch_cfg<Cfg16>(p, maps, pdl, stream);
+    case 16: return many_caches(p.C) ? launch_cfg<Cfg16Many>(p, maps, pdl, stream) : launch_cfg<Cfg16>(p, maps, pdl, stream);
     case 32: return launch_cfg<Cfg32>(p, maps, pdl, stream);
     case 48: return launch_cfg<Cfg48>(p, maps, pdl, stream);
     case 64: return launch_cfg<Cfg64>(p, maps, pdl, stream);
