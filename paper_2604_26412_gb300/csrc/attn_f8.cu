@@ -102,6 +102,8 @@ struct Cfg {
   static constexpr int kRows = kWarpRows * RG;  // rows per unit
   // Q^T fragments: in registers for 8 rows, else in shared memory (a piece's 32 registers of them spill)
   static constexpr bool kQSmem = NR > 1;
+  // The next unit's q is loaded while this one is computed, where the registers for it are free.
+  static constexpr bool kQAhead = NR == 2 && RG == 1;
   static constexpr int kQBytes = kQSmem ? RG * 8 * NR * 32 * 8 : 0;
 };
 
@@ -341,6 +343,22 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
     if constexpr (CF::kQSmem) return qf[(kstep * NR + nr) * 32];
     else return qreg[kstep];
   };
+  // This lane's part of a unit's q: of rows g (+ 8 nr), dims 32 q4 + 8 v .. + 7, the chunks v shared out over the key slices.
+  constexpr int kQV = CF::kQSmem ? 4 / CF::kKS : 4;
+  uint4 qw[NR][kQV];
+  auto load_q = [&](int c, int hr) {
+    const int qh = hr / p.row_blocks, qb = hr - qh * p.row_blocks;
+#pragma unroll
+    for (int nr = 0; nr < NR; ++nr) {
+      const int rr = qb * p.rows_per_unit + rg * CF::kWarpRows + 8 * nr + g;
+      const bool ok = rr < p.rows_total;
+      const int nl = ok ? rr / p.G : 0, gh = ok ? rr - nl * p.G : 0;
+      const uint4* src = reinterpret_cast<const uint4*>(
+          p.q + ((static_cast<size_t>(c) * p.Nq + nl) * p.hq + qh * p.G + gh) * kHeadDim + 32 * q4);
+#pragma unroll
+      for (int i = 0; i < kQV; ++i) qw[nr][i] = ok ? src[CF::kQSmem ? ks * kQV + i : i] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
   float o[8][NR][4];
   float m_run[NR][2], l_run[NR][2];  // rows 8 nr + 2 q4 + e; l_run: this lane's keys only
   int stage = 0;
@@ -355,26 +373,21 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
       h = cu.hr / p.row_blocks;
       rb = cu.hr - h * p.row_blocks;
       piece_lt0 = cu.lt;
+      if (!CF::kQAhead || cu.t == cu.t_begin) load_q(cu.c, cu.hr);
 #pragma unroll
       for (int nr = 0; nr < NR; ++nr) {
-        const int rl = rg * CF::kWarpRows + 8 * nr + g, rr = rb * p.rows_per_unit + rl;
-        const bool ok = rr < p.rows_total;
-        const int nl = ok ? rr / p.G : 0, gh = ok ? rr - nl * p.G : 0;
-        const uint4* src = reinterpret_cast<const uint4*>(
-            p.q + ((static_cast<size_t>(cu.c) * p.Nq + nl) * p.hq + h * p.G + gh) * kHeadDim + 32 * q4);
-        if (!CF::kQSmem || ks == 0) {
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {  // dims 32 q4 + 8 v .. + 7: k-steps 2 v, 2 v + 1
-            const uint4 w = ok ? src[v] : make_uint4(0u, 0u, 0u, 0u);
-            const uint2 f0 = make_uint2(bf16x2_to_f16x2(w.x), bf16x2_to_f16x2(w.y));
-            const uint2 f1 = make_uint2(bf16x2_to_f16x2(w.z), bf16x2_to_f16x2(w.w));
-            if constexpr (CF::kQSmem) {
-              qf[(2 * v * NR + nr) * 32] = f0;
-              qf[((2 * v + 1) * NR + nr) * 32] = f1;
-            } else {
-              qreg[2 * v] = f0;
-              qreg[2 * v + 1] = f1;
-            }
+        for (int i = 0; i < kQV; ++i) {
+          const int v = CF::kQSmem ? ks * kQV + i : i;  // k-steps 2 v, 2 v + 1
+          const uint4 w = qw[nr][i];
+          const uint2 f0 = make_uint2(bf16x2_to_f16x2(w.x), bf16x2_to_f16x2(w.y));
+          const uint2 f1 = make_uint2(bf16x2_to_f16x2(w.z), bf16x2_to_f16x2(w.w));
+          if constexpr (CF::kQSmem) {
+            qf[(2 * v * NR + nr) * 32] = f0;
+            qf[((2 * v + 1) * NR + nr) * 32] = f1;
+          } else {
+            qreg[2 * i] = f0;
+            qreg[2 * i + 1] = f1;
           }
         }
 #pragma unroll
@@ -383,6 +396,10 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
         l_run[nr][0] = l_run[nr][1] = 0.f;
       }
       o_codes = kWideV;
+      if (CF::kQAhead && cu.t + cu.ut - cu.lt < cu.t_end) {  // the next unit's
+        const bool same = cu.hr + 1 < HR;
+        load_q(same ? cu.c : cu.c + 1, same ? cu.hr + 1 : 0);
+      }
       if constexpr (CF::kQSmem) named_barrier_sync(kBarConsumers, CF::kWarps * 32);  // Q^T is shared by the key slices
     }
     if (ti.draft && p.tree) {
@@ -407,6 +424,8 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
 #pragma unroll 1
     for (int kw = ks * CF::kKW; kw < ks * CF::kKW + CF::kKW; kw += kChunk) {
       if (!live || kw >= ti.nkeys) break;
+      // Else the chunk's second 16 keys are draft keys that are all masked.  (64 rows: the branches cost more.)
+      const bool wide = CF::kRG >= 4 || codes || ti.nkeys > kw + 16;
       // S^T = K Q^T for 32 keys: s[m][nr][2 a + e] is key kw + 16 m + 8 a + g, row 8 nr + 2 q4 + e.
       float s[2][NR][4];
 #pragma unroll
@@ -447,6 +466,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
               else q = c8 == 0 ? qreg[st] : c8 == 1 ? qreg[2 + st] : c8 == 2 ? qreg[4 + st] : qreg[6 + st];
 #pragma unroll
               for (int m = 0; m < 2; ++m) {
+                if (m == 1 && !wide) break;
                 const uint4 &x = w[2 * m], &y = w[2 * m + 1];
                 mma_f16(s[m][nr], bf16x2_to_f16x2(word(x, 2 * st)), bf16x2_to_f16x2(word(y, 2 * st)),
                         bf16x2_to_f16x2(word(x, 2 * st + 1)), bf16x2_to_f16x2(word(y, 2 * st + 1)), q.x, q.y);
@@ -519,6 +539,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
       // O^T += V^T P^T, 16 keys per step.
 #pragma unroll
       for (int kk = 0; kk < 2; ++kk) {
+        if (kk == 1 && !wide) break;
         const int k0 = kw + 16 * kk;
         if (codes) {
           const uint32_t av = vbase + k0 * 128;
@@ -619,14 +640,18 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
 // Up to 8 rows, up to 16, 32, 48, 64.  What a CTA holds decides how many warps hide the latencies of
 // loads, conversions and the softmax: 8 rows fit three CTAs per SM (128 registers; two stages each: 105 us
 // per ragged-chain call of 64 caches against 117 us for two CTAs of three stages), 16 rows two (three would
-// spill).  Before this kernel the same calls took 185 us (4 rows) and 265 us (16 rows, 16 caches x 32K keys,
-// now 178 us): 64-key tiles, query rows as the MMA's M, 18.4 M instead of 13.1 M warp instructions per call of
+// spill).  48 rows take two key slices: with four, 13 warps are capped at 128 registers and spill (16 caches of 4096 tokens
+// 101 us per call, now 85).  Before this kernel the same calls took 185 us (4 rows) and 265 us (16 rows, 16 caches x 32K
+// keys, now 176 us): 64-key tiles, query rows as the MMA's M, 18.4 M instead of 13.1 M warp instructions per call of
 // 16 caches x 4096 tokens at 16 rows.
+// Short units are bound by what a unit costs beside its tiles: q is converted by all key slices, one unit ahead, and
+// the masked half of a draft chunk is left out (64 caches of 1024 tokens, 16 rows 59.7 -> 55.8 us per call, 4 rows 36.7 ->
+// 35.3).
 using Cfg8 = Cfg<1, 1, 4, 2, 3>;
 using Cfg16 = Cfg<2, 1, 4, 3, 2>;
 using Cfg16Many = Cfg<2, 1, 4, 2, 2>;
 using Cfg32 = Cfg<2, 2, 4, 5, 1>;
-using Cfg48 = Cfg<2, 3, 4, 5, 1>;
+using Cfg48 = Cfg<2, 3, 2, 5, 1>;
 using Cfg64 = Cfg<2, 4, 2, 5, 1>;
 
 // Every plan that kMaxCaches allows fits an SM.
