@@ -135,6 +135,7 @@ constexpr int kAppendCtas = 512;
 constexpr int kAppendSplits = 4;
 constexpr int kAppendGroup = 2;
 constexpr int kNormSplitNodes = 700;
+constexpr int kNormOverlapNodes = 384;
 
 __device__ __noinline__ void sincos_far(double theta, double* sn, double* cs) { sincos(theta, sn, cs); }
 
@@ -370,66 +371,51 @@ __global__ void __launch_bounds__(kAppendThreads, 5) append_kernel(const __grid_
 
 // QK-norm variant (Qwen3's per-head RMSNorm of q and k before RoPE): one warp per head, lane l
 // holding dims 2l, 2l + 1 and their RoPE partners + 64.  x <- x / sqrt(mean(x^2) + eps) * w (w the
-// head-dim weights), then the rotation; fp32 throughout, one rounding to bf16.
+// head-dim weights), then the rotation; fp32 throughout, one rounding to bf16.  One node to a CTA, shared out over
+// gridDim.y CTAs when there are few.  Latency bound, and a loop without loads ahead of it fits 32 registers, so sixteen
+// CTAs to an SM hide it: per call, 768 nodes of 32 + 8 heads 11.2 -> 8.3 us, 1024 nodes of 64 + 8 heads 17.4 -> 13.0
+// against the next head's loads, the weights' and V's ahead of the angles in 48 registers (9.3 and 15.8 us with fp64
+// angles and a CTA per node).
 __global__ void __launch_bounds__(kAppendThreads) append_qknorm_kernel(const __grid_constant__ AppendParams a) {
   begin_after_previous();
   __shared__ float s_cos[kHeadDim / 2], s_sin[kHeadDim / 2];
   const int heads = a.hq + a.hkv, h0 = share(heads, blockIdx.y), h1 = share(heads, blockIdx.y + 1);
   const int lane = threadIdx.x & 31, j = 2 * lane;
-  const int node0 = blockIdx.x * a.group, node1 = min(a.C * a.n_new, node0 + a.group);
-  int had = -1;
-  for (int node = node0; node < node1; ++node) {
-    const AppendNode t = append_node(a, node);
-    const int pos = a.positions[t.row];
-    auto source = [&](int hd) {
-      return (hd < a.hq ? a.q_in + (t.row * a.hq + hd) * kHeadDim : a.k_in + (t.row * a.hkv + hd - a.hq) * kHeadDim) + j;
-    };
-    int head = h0 + (threadIdx.x >> 5);
-    uint32_t lo = 0, hi = 0;
-    if (head < h1) {
-      lo = *reinterpret_cast<const uint32_t*>(source(head));
-      hi = *reinterpret_cast<const uint32_t*>(source(head) + 64);
-    }
-    append_v(a, t);
-    if (node == node0 || pos != had) {
-      if (node != node0) __syncthreads();
-      if (threadIdx.x < kHeadDim / 2) {
-        Pair sn, cs;
-        sincos_pair(static_cast<double>(pos) * a.inv_freq[threadIdx.x], &sn, &cs);
-        s_cos[threadIdx.x] = cs.h + cs.l;
-        s_sin[threadIdx.x] = sn.h + sn.l;
-      }
-      __syncthreads();
-      had = pos;
-    }
-    const float c0 = s_cos[j], s0 = s_sin[j], c1 = s_cos[j + 1], s1 = s_sin[j + 1];
-    while (head < h1) {
-      __nv_bfloat16* dst =
-          head < a.hq ? a.q_out + (t.row * a.hq + head) * kHeadDim
-                      : a.draft_k + ((static_cast<size_t>(t.c) * a.hkv + head - a.hq) * a.n_max + a.n0 + t.i) * kHeadDim;
-      const __nv_bfloat16* w = head < a.hq ? a.q_norm_w : a.k_norm_w;
-      const uint32_t wl = *reinterpret_cast<const uint32_t*>(w + j);
-      const uint32_t wh = *reinterpret_cast<const uint32_t*>(w + 64 + j);
-      float x[4] = {bf16_lo(lo), bf16_hi(lo), bf16_lo(hi), bf16_hi(hi)};
-      head += kAppendThreads / 32;
-      if (head < h1) {  // the warp's next head
-        lo = *reinterpret_cast<const uint32_t*>(source(head));
-        hi = *reinterpret_cast<const uint32_t*>(source(head) + 64);
-      }
-      float ss = x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-      const float r = rsqrtf(ss * (1.f / kHeadDim) + a.eps);
-      x[0] *= r * bf16_lo(wl);
-      x[1] *= r * bf16_hi(wl);
-      x[2] *= r * bf16_lo(wh);
-      x[3] *= r * bf16_hi(wh);
-      const float y0 = x[0] * c0 - x[2] * s0, y1 = x[1] * c1 - x[3] * s1;   // dims j, j + 1
-      const float z0 = x[2] * c0 + x[0] * s0, z1 = x[3] * c1 + x[1] * s1;   // dims j + 64, j + 65
-      *reinterpret_cast<uint32_t*>(dst + j) = pack_bf16x2(y0, y1);
-      *reinterpret_cast<uint32_t*>(dst + 64 + j) = pack_bf16x2(z0, z1);
-    }
+  const AppendNode t = append_node(a, blockIdx.x);
+  const int pos = a.positions[t.row];
+  if (threadIdx.x < kHeadDim / 2) {
+    Pair sn, cs;
+    sincos_pair(static_cast<double>(pos) * a.inv_freq[threadIdx.x], &sn, &cs);
+    s_cos[threadIdx.x] = cs.h + cs.l;
+    s_sin[threadIdx.x] = sn.h + sn.l;
   }
+  __syncthreads();
+  for (int head = h0 + (threadIdx.x >> 5); head < h1; head += kAppendThreads / 32) {
+    const bool query = head < a.hq;
+    const __nv_bfloat16* src = (query ? a.q_in + (t.row * a.hq + head) * kHeadDim : a.k_in + (t.row * a.hkv + head - a.hq) * kHeadDim) + j;
+    __nv_bfloat16* dst =
+        query ? a.q_out + (t.row * a.hq + head) * kHeadDim
+              : a.draft_k + ((static_cast<size_t>(t.c) * a.hkv + head - a.hq) * a.n_max + a.n0 + t.i) * kHeadDim;
+    const __nv_bfloat16* w = query ? a.q_norm_w : a.k_norm_w;
+    const uint32_t lo = *reinterpret_cast<const uint32_t*>(src), hi = *reinterpret_cast<const uint32_t*>(src + 64);
+    const uint32_t wl = *reinterpret_cast<const uint32_t*>(w + j);
+    const uint32_t wh = *reinterpret_cast<const uint32_t*>(w + 64 + j);
+    float x[4] = {bf16_lo(lo), bf16_hi(lo), bf16_lo(hi), bf16_hi(hi)};
+    float ss = x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    const float r = rsqrtf(ss * (1.f / kHeadDim) + a.eps);
+    x[0] *= r * bf16_lo(wl);
+    x[1] *= r * bf16_hi(wl);
+    x[2] *= r * bf16_lo(wh);
+    x[3] *= r * bf16_hi(wh);
+    const float c0 = s_cos[j], s0 = s_sin[j], c1 = s_cos[j + 1], s1 = s_sin[j + 1];
+    const float y0 = x[0] * c0 - x[2] * s0, y1 = x[1] * c1 - x[3] * s1;   // dims j, j + 1
+    const float z0 = x[2] * c0 + x[0] * s0, z1 = x[3] * c1 + x[1] * s1;   // dims j + 64, j + 65
+    *reinterpret_cast<uint32_t*>(dst + j) = pack_bf16x2(y0, y1);
+    *reinterpret_cast<uint32_t*>(dst + 64 + j) = pack_bf16x2(z0, z1);
+  }
+  append_v(a, t);
 }
 
 }  // namespace
@@ -454,14 +440,16 @@ cudaError_t launch_append(AppendParams a, cudaStream_t stream) {
   const int nodes = a.C * a.n_new;
   const bool norm = a.q_norm_w != nullptr;
   int splits = std::min(kAppendSplits, kAppendCtas / nodes);
-  // With QK-norm the angles weigh less: two CTAs to a node up to 700 nodes (64 caches of 7 nodes, with the attention
-  // behind it, 56.8 -> 55.0 us; 768 nodes 58.1 against 58.8), and never two nodes to a CTA, whose longer CTAs made a
-  // second wave (1540 nodes 20.5 -> 13.9 us).
+  // With QK-norm the angles weigh less: two CTAs to a node up to 700 nodes (steps of 64 caches with 7 nodes a level 133.9
+  // -> 130.8 us; beyond, 768 nodes alone 9.0 against 8.3), and one node to a CTA at any number.
   if (norm) splits = std::max(splits, std::min(2, kNormSplitNodes / nodes * 2));
   splits = std::max(1, splits);
   a.group = norm ? 1 : std::max(1, std::min(kAppendGroup, nodes / kAppendCtas));
+  // Launched behind its predecessor; with QK-norm only up to 384 nodes, from where the CTAs that wait cost more than the
+  // launch (steps of 64 caches with 7 nodes a level 134.9 us, 130.8 without; 1 cache with 4 nodes a level 38.0, 36.7 with).
   return launch_maybe_pdl(norm ? append_qknorm_kernel : append_kernel,
-                          dim3((nodes + a.group - 1) / a.group, splits), dim3(kAppendThreads), 0, true, stream, a);
+                          dim3((nodes + a.group - 1) / a.group, splits), dim3(kAppendThreads), 0,
+                          !norm || nodes <= kNormOverlapNodes, stream, a);
 }
 
 }  // namespace kvshot

@@ -70,6 +70,15 @@ def test_qknorm_append_matches_oracle(C, hq, hkv, n_new, n0, n_max, max_pos):
     _case(C, hq, hkv, n_new, n0, n_max, max_pos, seed=C * 1000 + n_new)
 
 
+# The grids: four, two and one CTA to a node (128, 129, 700, 701 nodes), launched behind the predecessor and not (384,
+# 385), heads and V chunks that the CTAs of a node do not divide, fewer heads than CTAs' warps.
+@pytest.mark.parametrize("C,n_new,hq,hkv", [
+    (8, 16, 32, 8), (3, 43, 5, 1), (4, 50, 9, 3), (6, 64, 6, 2), (5, 77, 10, 5), (10, 50, 32, 8), (10, 70, 3, 1),
+    (1, 701, 5, 5), (30, 50, 6, 2)])
+def test_qknorm_append_grids(C, n_new, hq, hkv):
+    _case(C, hq, hkv, n_new, 1, n_new + 2, 40000, seed=C + n_new)
+
+
 def test_qknorm_append_in_place():
     _case(2, 32, 8, 6, 1, 8, 30000, seed=11, in_place=True)
 
