@@ -333,10 +333,6 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 }  // namespace
 
-int attn_cc_ctas_per_sm() { return 2; }
-
-size_t attn_cc_smem_bytes(int C) { return smem_bytes(C); }
-
 cudaError_t attn_cc_occupancy(int C, int* ctas_per_sm) {
   const size_t smem = smem_bytes(C);
   cudaError_t e = cudaFuncSetAttribute(attn_cc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -424,8 +424,6 @@ cudaError_t occupancy_cfg(int C, int* ctas) {
 
 }  // namespace
 
-int attn_mma_ctas_per_sm(int m_tiles) { return m_tiles == 1 ? Cfg1<false>::kMinBlocks : 1; }
-
 cudaError_t attn_mma_occupancy(int m_tiles, int C, int* ctas_per_sm) {
   switch (m_tiles) {
     case 1: return occupancy_cfg<Cfg1<false>>(C, ctas_per_sm);

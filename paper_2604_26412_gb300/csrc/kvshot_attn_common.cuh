@@ -530,30 +530,19 @@ struct Pipe {
   int* issued;         // tiles issued by the producer
 };
 
-// q staging (tensor-memory kernel only): piece k's query block goes to buffer
-// k % nbuf (two 64-dim halves of 128 rows, 128B-swizzled).
-struct QPipe {
-  uint8_t* buf;        // nbuf x kQBufBytes, 1024-aligned
-  uint64_t* full;      // [nbuf] TMA -> MMA issuer
-  uint64_t* empty;     // [nbuf] MMA completion -> TMA
-  int nbuf;            // q buffers (piece k uses buffer k % nbuf)
-  int rows;            // rows loaded per box (G x nodes per box)
-  int nq_box;          // draft nodes per box
-  int* issued;         // q blocks issued
-};
+// The tensor-memory kernel's staged query block: two 64-dim halves of 128 rows, 128B-swizzled.
 constexpr int kQRows = 128;
 constexpr int kQBufBytes = 2 * kQRows * 128;
 
 // The producer warp: walks this CTA's tiles and issues their TMA loads into the
 // stage ring, one tile ahead on the page-table reads.  Lane 0 issues.
 __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMaps& maps, const Pipe& pipe, const int* s_len,
-                             Cursor cu, const QPipe* qp = nullptr) {
+                             Cursor cu) {
   const int lane = threadIdx.x & 31;
   const uint64_t policy = l2_policy_evict_first();
   int stage = 0;
   uint32_t phase = 0;
   int issued = 0;
-  int piece = 0;
   bool waited = false;  // griddepcontrol.wait done
   // Several units per CTA: each is a few tiles, so the first unit's, loaded beside the preceding kernel, are a small
   // part of the call's and slow that kernel more than they save (220 caches of 41..83 tokens: 55.3 us per level,
@@ -582,29 +571,7 @@ __device__ __forceinline__ void run_producer(const AttnParams& p, const TensorMa
     }
 
     int ok = 1;
-    if (qp != nullptr && (cu.t == cu.t_begin || cu.lt == 0)) {
-      // First tile of a piece: stage the unit's query block (all its G x Nq rows).
-      if (lane == 0) {
-        const int qb = piece % qp->nbuf;
-        const uint32_t qbar = smem_addr(&qp->full[qb]);
-        ok = mbar_wait(smem_addr(&qp->empty[qb]), ((piece / qp->nbuf) & 1) ^ 1u, p.err, p.wait_ns) ? 1 : 0;
-        if (ok && !*pipe.abort) {
-          const int rb = cu.hr - h * p.row_blocks;
-          const uint32_t dst = smem_addr(qp->buf + qb * kQBufBytes);
-          mbar_arrive_expect_tx(qbar, 2 * qp->rows * 128);
-          tma_load_4d(dst, &maps.q, 0, h * p.G, rb * qp->nq_box, cu.c, qbar);
-          tma_load_4d(dst + kQRows * 128, &maps.q, 64, h * p.G, rb * qp->nq_box, cu.c, qbar);
-          *qp->issued = piece + 1;
-        } else {
-          ok = 0;
-        }
-      }
-      ++piece;
-    }
-    if (lane == 0 && ok) {
-      ok = mbar_wait(smem_addr(&pipe.empty[stage]), phase ^ 1u, p.err, p.wait_ns) ? 1 : 0;
-      if (!ok || *pipe.abort) ok = 0;
-    }
+    if (lane == 0) ok = mbar_wait(smem_addr(&pipe.empty[stage]), phase ^ 1u, p.err, p.wait_ns) && !*pipe.abort;
     ok = __shfl_sync(0xffffffffu, ok, 0);
     if (!ok) {
       if (lane == 0) *pipe.abort = 1;

@@ -152,9 +152,4 @@ cudaError_t launch_maybe_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, siz
 cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream);
 cudaError_t launch_append(AppendParams a, cudaStream_t stream);  // with QK-norm when a.q_norm_w is set
 
-// CTAs per SM each kernel variant is built for (its shared-memory ring and
-// register budget are sized for this residency).
-int attn_cc_ctas_per_sm();
-int attn_mma_ctas_per_sm(int m_tiles);
-
 }  // namespace kvshot
