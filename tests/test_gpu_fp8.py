@@ -226,6 +226,27 @@ def test_fp8_largest_number_of_caches(nq, hq, hkv):
     gh.compare(out[some], lse[some], ref_out, ref_lse, f"fp8 1024 caches nq={nq} {hq}/{hkv}")
 
 
+# 256 rows over as many units as put 128-row blocks (912 + 152 of them) past the library's own scratch: 64-row blocks, which
+# fit it, run there, with a workspace and with that scratch; 53 caches keep the 128-row blocks.
+@pytest.mark.parametrize("caches", [53, 57])
+def test_fp8_blocks_at_the_limit_of_the_static_scratch(caches):
+    case = ([(29 * c) % 140 for c in range(caches)], (8, 12, 12, 12, 12, 8), True, True, 16, 32, 8, 64)
+    spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(case, seed=caches)
+    some = [0, 1, 30, caches - 1]
+    ref_out, ref_lse = gh.oracle_attn(hc, q, dk, dv, N, Nq, caches=some)
+    out, lse = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
+    gh.compare(out[some], lse[some], ref_out, ref_lse, f"fp8 {caches} caches")
+    d = kvshot.make_desc(num_caches=caches, num_seqs=caches, hq=32, hkv=8, n_nodes=N, n_query=Nq, n_max=inp.n_max,
+                         max_seq_len=spec.max_seq_len, page_size=16, max_pages_per_seq=inp.page_table.shape[1],
+                         num_pages=inp.num_pages, tree=True, flags=kvshot.KVSHOT_TARGET_FP8,
+                         k_scale_exp=wl.FP8_K_EXP, v_scale_exp=wl.FP8_V_EXP)
+    assert kvshot.workspace_size(d) <= 64 << 20
+    assert kvshot.draft_attn_static_status(d, q, tk8, tv8, inp.page_table, inp.seq_lens, dk, dv, inp.tree_parent, out,
+                                           lse) == kvshot.KVSHOT_OK
+    torch.cuda.synchronize()
+    gh.compare(out[some], lse[some], ref_out, ref_lse, f"fp8 {caches} caches, static scratch")
+
+
 def test_fp8_is_deterministic_and_differs_from_bf16_only_by_quantisation():
     spec, inp, dk, dv, q, N, Nq, tk8, tv8, hc = _setup(((2000, 900), (4, 4), True, True, 16, 32, 8, 4), seed=21)
     a = _run(spec, inp, tk8, tv8, dk, dv, q, N, Nq, 0)
