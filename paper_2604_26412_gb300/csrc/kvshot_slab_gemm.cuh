@@ -54,6 +54,11 @@ constexpr int kRingBytes = 200 * 1024;
 constexpr uint32_t kTmemCols = 512;         // two accumulators of N <= 256 columns
 constexpr int kMaxN = 256;                  // the MMA's largest N
 constexpr int kMaxEntries = 4;
+// Limit on a wait of the pipeline.  (tests/test_gpu_fusion.py builds copies in which both CTAs of a pair, or one, give up
+// at once.)
+#ifndef KVSHOT_FUSION_WAIT_NS
+#define KVSHOT_FUSION_WAIT_NS kWaitLimitNs
+#endif
 
 struct Entry {
   int8_t w;    // weight map index
@@ -81,6 +86,13 @@ struct Maps {
 };
 
 inline size_t smem_bytes() { return 1024 + kRingBytes + 8 * (2 * kMaxStages + 1) + 16; }
+
+__device__ __forceinline__ void store_in_pair(uint32_t addr, int rank, int v) {
+  asm volatile("{\n\t.reg .u32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\tst.shared::cluster.s32 [ra], %2;\n\t}" ::"r"(
+                   addr),
+               "r"(rank), "r"(v)
+               : "memory");
+}
 
 __device__ __forceinline__ void pair_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -127,6 +139,7 @@ __global__ void __launch_bounds__(kThreads, 1) slab_gemm(const __grid_constant__
   uint64_t* done = empty + kMaxStages;
   uint32_t* tmem_base = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* gave_up = reinterpret_cast<volatile int*>(tmem_base + 1);
+  volatile int* peer = gave_up + 1;  // written by the pair's other CTA: k-tiles issued, or -1 - that where it gave up
   if (threadIdx.x == 0) {
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_addr(&full[s]), 1);
@@ -155,27 +168,31 @@ __global__ void __launch_bounds__(kThreads, 1) slab_gemm(const __grid_constant__
   const int nk = p.nk;
   bool ok = true;
   int issued = 0;
+  const uint64_t stream_once = l2_policy_evict_first();  // weights: read once
+  const uint32_t tx = 2u * static_cast<uint32_t>(slot);  // both CTAs' bytes (rows out of range are filled)
+  const int ty = tt * p.box_tok, half = N / 2;
+  const uint32_t even0 = in_even_cta(smem_addr(full)), ring = smem_addr(base);
+  auto load = [&](int kt, int s) {
+    if (rank == 0) mbar_arrive_expect_tx(smem_addr(&full[s]), tx);
+    const uint32_t fb = even0 + 8 * s, dst = ring + s * slot, bdst = dst + kABytes;
+    tma_load_pair_hint(dst, &maps.w[en.w], en.wx0 + kt * kKT, f0, fb, stream_once);
+    if (stacked) {
+      const CUtensorMap* a = &maps.a[rank ? en.a1 : en.a0];
+      tma_load_pair(bdst, a, kt * kKT, ty, fb);
+      tma_load_pair(bdst + btile, a, kt * kKT, ty + half, fb);
+    } else {
+      tma_load_pair(bdst, &maps.a[en.a0], kt * kKT, ty + rank * half, fb);
+      if (both) tma_load_pair(bdst + btile, &maps.a[en.a1], kt * kKT, ty + rank * half, fb);
+    }
+  };
   if (warp == 0 && lane == 0) {
-    const uint64_t stream_once = l2_policy_evict_first();  // weights: read once
-    const uint32_t tx = 2u * static_cast<uint32_t>(slot);  // both CTAs' bytes (rows out of range are filled)
-    const int ty = tt * p.box_tok, half = N / 2;
-    const uint32_t full0 = smem_addr(full), even0 = in_even_cta(full0), empty0 = smem_addr(empty), ring = smem_addr(base);
+    const uint32_t empty0 = smem_addr(empty);
     int s = 0;
     uint32_t phase = 1;  // of the empty barriers: their first use needs no wait
     for (int kt = 0; kt < nk; ++kt) {
-      if (kt >= nst) ok = mbar_wait(empty0 + 8 * s, phase, p.err);
+      if (kt >= nst) ok = mbar_wait(empty0 + 8 * s, phase, p.err, KVSHOT_FUSION_WAIT_NS);
       if (!ok) break;
-      if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, tx);
-      const uint32_t fb = even0 + 8 * s, dst = ring + s * slot, bdst = dst + kABytes;
-      tma_load_pair_hint(dst, &maps.w[en.w], en.wx0 + kt * kKT, f0, fb, stream_once);
-      if (stacked) {
-        const CUtensorMap* a = &maps.a[rank ? en.a1 : en.a0];
-        tma_load_pair(bdst, a, kt * kKT, ty, fb);
-        tma_load_pair(bdst + btile, a, kt * kKT, ty + half, fb);
-      } else {
-        tma_load_pair(bdst, &maps.a[en.a0], kt * kKT, ty + rank * half, fb);
-        if (both) tma_load_pair(bdst + btile, &maps.a[en.a1], kt * kKT, ty + rank * half, fb);
-      }
+      load(kt, s);
       issued = kt + 1;
       if (++s == nst) {
         s = 0;
@@ -195,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) slab_gemm(const __grid_constant__
       int s = 0;
       uint32_t phase = 0, acc = 0;
       for (int kt = 0; kt < nk; ++kt) {
-        ok = mbar_wait(full0 + 8 * s, phase, p.err);
+        ok = mbar_wait(full0 + 8 * s, phase, p.err, KVSHOT_FUSION_WAIT_NS);
         if (!ok) break;
         tc_fence_after();
         // Descriptors hold addresses in units of 16 bytes, and the whole ring stays below their 256 KB.
@@ -220,11 +237,9 @@ __global__ void __launch_bounds__(kThreads, 1) slab_gemm(const __grid_constant__
     tc_commit_pair(smem_addr(done));  // every MMA this thread issued has completed
   }
   __syncwarp();
-  ok = mbar_wait(smem_addr(done), 0, p.err);
+  ok = mbar_wait(smem_addr(done), 0, p.err, KVSHOT_FUSION_WAIT_NS);
+  if (!ok) *gave_up = 1;
   tc_fence_after();
-  if (rank == 0 && threadIdx.x == 0 && *gave_up)  // let the copies in flight land before the CTAs exit
-    for (int kt = max(0, issued - nst); kt < issued; ++kt)
-      mbar_wait(smem_addr(&full[kt % nst]), (kt / nst) & 1, p.err);
   const int f = f0 + warp * 32 + lane;
   const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
   float* slab = p.slab + static_cast<size_t>(z) * p.T * p.d_out;
@@ -247,7 +262,22 @@ __global__ void __launch_bounds__(kThreads, 1) slab_gemm(const __grid_constant__
   }
   tc_fence_before();
   __syncthreads();
+  const bool failed = *gave_up;
+  if (threadIdx.x == 0) store_in_pair(smem_addr(tmem_base + 2), rank ^ 1, failed ? -1 - issued : issued);
   pair_sync();  // the pair's MMAs and barriers are used across the two CTAs until here
+  if (failed || *peer < 0) {
+    // The copies in flight land, and the MMAs end, before the CTAs exit.  A k-tile that one CTA alone has loaded would
+    // never complete its barrier, so the other loads it too (no MMA reads the ring any more).
+    if (threadIdx.x == 0) {
+      const int other = *peer, last = max(issued, other < 0 ? -1 - other : other);
+      mbar_wait(smem_addr(done), 0, p.err);
+      for (int kt = issued; kt < last; ++kt) load(kt, kt % nst);
+      for (int kt = max(0, last - nst); rank == 0 && kt < last; ++kt)
+        mbar_wait(smem_addr(&full[kt % nst]), (kt / nst) & 1, p.err);
+    }
+    __syncthreads();
+    pair_sync();
+  }
   if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);
 }
 

@@ -6,11 +6,17 @@ products: relative error ~1e-6) and rounds h once to bf16 (at most 2^-9 of
 bf16 ulp plus the fp32 accumulation), and the relative L2 error over the
 output must be <= 3e-3.
 """
+import ctypes
+import glob
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
 from oracle import fusion as fo
+from paper_2604_26412_gb300 import build
 from paper_2604_26412_gb300 import kvshot
 from paper_2604_26412_gb300 import workloads as wl
 
@@ -104,3 +110,31 @@ def test_workspace_reuse_and_garbage():
     for T, d in shapes:
         fi = wl.fusion_inputs(T, d, device="cuda", seed=T)
         _compare(_run(fi, T, d, ws=ws), _oracle(fi), f"reused workspace T={T} d={d}")
+
+
+# Copies of the library whose pipeline waits give up at once in both CTAs of a pair, in the odd one (the other then loads
+# k-tiles that it does not, and waits its full two seconds for them) and in the even one: the call ends and records the
+# timeout, and the next call of the ordinary library is correct.
+@pytest.mark.parametrize("limit", ["1", "(blockIdx.x & 1 ? 1 : kWaitLimitNs)", "(blockIdx.x & 1 ? kWaitLimitNs : 1)"])
+def test_a_call_that_times_out_ends(limit, tmp_path):
+    obj, lib_path = str(tmp_path / "gated_delta.o"), str(tmp_path / "libkvshot_impatient.so")
+    kvshot.load()
+    others = [o for o in glob.glob(os.path.join(build.BUILD, "*.o")) if not o.endswith("gated_delta.o")]
+    subprocess.run([build.nvcc(), *build.ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", build.INCLUDE,
+                    f"-DKVSHOT_FUSION_WAIT_NS={limit}", "-c", os.path.join(build.CSRC, "gated_delta.cu"), "-o", obj],
+                   check=True)
+    subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-o", lib_path, obj, *others], check=True)
+    impatient = ctypes.CDLL(lib_path).kvshot_gated_delta
+    impatient.argtypes, impatient.restype = kvshot.load().kvshot_gated_delta.argtypes, ctypes.c_int
+    for T, d in ((1, 1024), (192, 2048)):
+        fi = wl.fusion_inputs(T, d, device="cuda", seed=T)
+        desc = kvshot.make_fusion_desc(num_tokens=T, hidden=d)
+        ws = torch.empty(kvshot.gated_delta_workspace_size(desc), dtype=torch.uint8, device="cuda")
+        err = torch.zeros(1, dtype=torch.int32, device="cuda")
+        desc.workspace, desc.workspace_bytes, desc.err_flag = ws.data_ptr(), ws.numel(), err.data_ptr()
+        h = torch.empty((T, d), dtype=torch.bfloat16, device="cuda")
+        assert impatient(ctypes.byref(desc), *(t.data_ptr() for t in (fi.n, fi.o, fi.w_g, fi.b_g, fi.w_delta, h)),
+                         torch.cuda.current_stream().cuda_stream) == kvshot.KVSHOT_OK
+        torch.cuda.synchronize()
+        assert int(err.item()) == kvshot.KVSHOT_ERR_TIMEOUT
+        _compare(_run(fi, T, d), _oracle(fi), f"after a timed-out call, T={T} d={d}")
