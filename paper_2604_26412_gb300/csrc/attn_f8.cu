@@ -32,6 +32,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "kvshot_attn_common.cuh"
 
@@ -102,8 +103,7 @@ struct Cfg {
   static constexpr int kRows = kWarpRows * RG;  // rows per unit
   // Q^T fragments: in registers for 8 rows, else in shared memory (a piece's 32 registers of them spill)
   static constexpr bool kQSmem = NR > 1;
-  // The next unit's q is loaded while this one is computed, where the registers for it are free.
-  static constexpr bool kQAhead = NR == 2 && RG == 1;
+  static constexpr bool kDraftRows = NR == 2 && RG < 4;  // two key slices share a draft tile's keys, each for half of the rows
   static constexpr int kQBytes = kQSmem ? RG * 8 * NR * 32 * 8 : 0;
 };
 
@@ -343,22 +343,6 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
     if constexpr (CF::kQSmem) return qf[(kstep * NR + nr) * 32];
     else return qreg[kstep];
   };
-  // This lane's part of a unit's q: of rows g (+ 8 nr), dims 32 q4 + 8 v .. + 7, the chunks v shared out over the key slices.
-  constexpr int kQV = CF::kQSmem ? 4 / CF::kKS : 4;
-  uint4 qw[NR][kQV];
-  auto load_q = [&](int c, int hr) {
-    const int qh = hr / p.row_blocks, qb = hr - qh * p.row_blocks;
-#pragma unroll
-    for (int nr = 0; nr < NR; ++nr) {
-      const int rr = qb * p.rows_per_unit + rg * CF::kWarpRows + 8 * nr + g;
-      const bool ok = rr < p.rows_total;
-      const int nl = ok ? rr / p.G : 0, gh = ok ? rr - nl * p.G : 0;
-      const uint4* src = reinterpret_cast<const uint4*>(
-          p.q + ((static_cast<size_t>(c) * p.Nq + nl) * p.hq + qh * p.G + gh) * kHeadDim + 32 * q4);
-#pragma unroll
-      for (int i = 0; i < kQV; ++i) qw[nr][i] = ok ? src[CF::kQSmem ? ks * kQV + i : i] : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
   float o[8][NR][4];
   float m_run[NR][2], l_run[NR][2];  // rows 8 nr + 2 q4 + e; l_run: this lane's keys only
   int stage = 0;
@@ -373,13 +357,18 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
       h = cu.hr / p.row_blocks;
       rb = cu.hr - h * p.row_blocks;
       piece_lt0 = cu.lt;
-      if (!CF::kQAhead || cu.t == cu.t_begin) load_q(cu.c, cu.hr);
+      constexpr int kQV = CF::kQSmem ? 4 / CF::kKS : 4;  // chunks of 8 dims of each lane's 32: the key slices share them
 #pragma unroll
       for (int nr = 0; nr < NR; ++nr) {
+        const int rr = rb * p.rows_per_unit + rg * CF::kWarpRows + 8 * nr + g;
+        const bool ok = rr < p.rows_total;
+        const int nl = ok ? rr / p.G : 0, gh = ok ? rr - nl * p.G : 0;
+        const uint4* src = reinterpret_cast<const uint4*>(
+            p.q + ((static_cast<size_t>(cu.c) * p.Nq + nl) * p.hq + h * p.G + gh) * kHeadDim + 32 * q4);
 #pragma unroll
         for (int i = 0; i < kQV; ++i) {
-          const int v = CF::kQSmem ? ks * kQV + i : i;  // k-steps 2 v, 2 v + 1
-          const uint4 w = qw[nr][i];
+          const int v = CF::kQSmem ? ks * kQV + i : i;  // dims 32 q4 + 8 v .. + 7: k-steps 2 v, 2 v + 1
+          const uint4 w = ok ? src[v] : make_uint4(0u, 0u, 0u, 0u);
           const uint2 f0 = make_uint2(bf16x2_to_f16x2(w.x), bf16x2_to_f16x2(w.y));
           const uint2 f1 = make_uint2(bf16x2_to_f16x2(w.z), bf16x2_to_f16x2(w.w));
           if constexpr (CF::kQSmem) {
@@ -396,10 +385,6 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
         l_run[nr][0] = l_run[nr][1] = 0.f;
       }
       o_codes = kWideV;
-      if (CF::kQAhead && cu.t + cu.ut - cu.lt < cu.t_end) {  // the next unit's
-        const bool same = cu.hr + 1 < HR;
-        load_q(same ? cu.c : cu.c + 1, same ? cu.hr + 1 : 0);
-      }
       if constexpr (CF::kQSmem) named_barrier_sync(kBarConsumers, CF::kWarps * 32);  // Q^T is shared by the key slices
     }
     if (ti.draft && p.tree) {
@@ -418,21 +403,22 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
     const uint32_t kbase = smem_addr(pipe.ring + static_cast<size_t>(stage) * kStageBytes);
     const bool codes = !ti.draft;
     const uint32_t vbase = kbase + (codes ? kCodeBytes : kKVTileBytes);
-    const bool full = codes && ti.nkeys == kPK;  // every key of the tile is visible to every row
     // The key scale is part of the score scale, the value scale part of P (kWideV: of O); the sum keeps the unscaled P.
     const float qs = codes ? p.qscale * p.k_scale : p.qscale, vs = codes && !kWideV ? p.v_scale : 1.f;
-#pragma unroll 1
-    for (int kw = ks * CF::kKW; kw < ks * CF::kKW + CF::kKW; kw += kChunk) {
-      if (!live || kw >= ti.nkeys) break;
-      // Else the chunk's second 16 keys are draft keys that are all masked.  (64 rows: the branches cost more.)
-      const bool wide = CF::kRG >= 4 || codes || ti.nkeys > kw + 16;
+    // 32 keys of the tile from key kw on.  Draft chunks: 8-row step `only` alone (-1: all), and the second 16 keys
+    // only where one of them is visible.
+    auto chunk = [&](auto draft, int kw, int only) {
+      constexpr bool kDraft = decltype(draft)::value;
+      const bool full = !kDraft && ti.nkeys == kPK;  // every key of the tile is visible to every row
+      const bool wide = !kDraft || ti.nkeys > kw + 16;
+      auto skip = [&](int nr) { return kDraft && CF::kDraftRows && nr != only; };
       // S^T = K Q^T for 32 keys: s[m][nr][2 a + e] is key kw + 16 m + 8 a + g, row 8 nr + 2 q4 + e.
       float s[2][NR][4];
 #pragma unroll
       for (int m = 0; m < 2; ++m)
 #pragma unroll
         for (int nr = 0; nr < NR; ++nr) s[m][nr][0] = s[m][nr][1] = s[m][nr][2] = s[m][nr][3] = 0.f;
-      if (codes) {
+      if constexpr (!kDraft) {
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) {
           const uint32_t a = kbase + (kh ? koff1 : koff0) + kw * 128;
@@ -461,6 +447,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
           for (int st = 0; st < 2; ++st)
 #pragma unroll
             for (int nr = 0; nr < NR; ++nr) {
+              if (skip(nr)) continue;
               uint2 q;
               if constexpr (CF::kQSmem) q = q_frag(2 * c8 + st, nr);
               else q = c8 == 0 ? qreg[st] : c8 == 1 ? qreg[2 + st] : c8 == 2 ? qreg[4 + st] : qreg[6 + st];
@@ -483,8 +470,8 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int key = kw + 16 * m + 8 * (e >> 1) + g;
-              bool valid = key < ti.nkeys;
-              if (ti.draft)
+              bool valid = key < ti.nkeys && !skip(nr);
+              if (kDraft)
                 valid = valid && draft_visible(p, sm.anc, rb * p.rows_per_unit + rg * CF::kWarpRows + 8 * nr + 2 * q4 + (e & 1),
                                                ti.key0 + key);
               if (!valid) s[m][nr][e] = -INFINITY;
@@ -498,7 +485,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
           mx[nr][e] = fmaxf(fmaxf(s[0][nr][e], s[0][nr][2 + e]), fmaxf(s[1][nr][e], s[1][nr][2 + e])) * qs;
           grow |= mx[nr][e] > m_run[nr][e];
         }
-      const bool leave_codes = kWideV && !codes && o_codes;  // warp-uniform
+      const bool leave_codes = kWideV && kDraft && o_codes;  // warp-uniform
       if (__any_sync(0xffffffffu, grow || leave_codes)) {
 #pragma unroll
         for (int nr = 0; nr < NR; ++nr)
@@ -519,11 +506,12 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
             }
           }
       }
-      o_codes &= codes;
+      if (kDraft) o_codes = false;
       // P^T fragments of the chunk's two 16-key steps.
       uint32_t pb[2][NR][2];
 #pragma unroll
       for (int nr = 0; nr < NR; ++nr) {
+        if (skip(nr)) continue;
         const float m0 = m_run[nr][0] == -INFINITY ? 0.f : m_run[nr][0];
         const float m1 = m_run[nr][1] == -INFINITY ? 0.f : m_run[nr][1];
 #pragma unroll
@@ -541,7 +529,7 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
       for (int kk = 0; kk < 2; ++kk) {
         if (kk == 1 && !wide) break;
         const int k0 = kw + 16 * kk;
-        if (codes) {
+        if constexpr (!kDraft) {
           const uint32_t av = vbase + k0 * 128;
           uint4 w[4] = {lds128(av + voff0), lds128(av + voff1), lds128(av + voff0 + 1024), lds128(av + voff1 + 1024)};
           if (!full) {  // rows past the valid keys may hold NaN codes
@@ -580,11 +568,23 @@ __device__ __forceinline__ void run_consumer(const AttnParams& p, const Smem& sm
               const uint32_t a3 = bf16x2_to_f16x2(__byte_perm(cb, db, 0x7632));
 #pragma unroll
               for (int nr = 0; nr < NR; ++nr)
-                mma_f16(o[4 * hh + t][nr], a0, a1, a2, a3, pb[kk][nr][0], pb[kk][nr][1]);
+                if (!skip(nr)) mma_f16(o[4 * hh + t][nr], a0, a1, a2, a3, pb[kk][nr][0], pb[kk][nr][1]);
             }
           }
         }
       }
+    };
+    const int kw1 = min(ks * CF::kKW + CF::kKW, ti.nkeys);
+    if (live && codes) {
+#pragma unroll 1
+      for (int kw = ks * CF::kKW; kw < kw1; kw += kChunk) chunk(std::false_type{}, kw, -1);
+    } else if (live && CF::kDraftRows) {
+      // Two slices take the same draft keys for 8 rows each: few keys would leave one warp all the rows.
+#pragma unroll 1
+      for (int kw = (ks >> 1) * kChunk; kw < ti.nkeys; kw += CF::kKS / 2 * kChunk) chunk(std::true_type{}, kw, ks & 1);
+    } else if (live) {
+#pragma unroll 1
+      for (int kw = ks * CF::kKW; kw < kw1; kw += kChunk) chunk(std::true_type{}, kw, -1);
     }
     __syncwarp();
     if (live) {
@@ -644,9 +644,10 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
 // 101 us per call, now 85).  Before this kernel the same calls took 185 us (4 rows) and 265 us (16 rows, 16 caches x 32K
 // keys, now 176 us): 64-key tiles, query rows as the MMA's M, 18.4 M instead of 13.1 M warp instructions per call of
 // 16 caches x 4096 tokens at 16 rows.
-// Short units are bound by what a unit costs beside its tiles: q is converted by all key slices, one unit ahead, and
-// the masked half of a draft chunk is left out (64 caches of 1024 tokens, 16 rows 59.7 -> 55.8 us per call, 4 rows 36.7 ->
-// 35.3).
+// Short units are bound by what a unit costs beside its tiles.  q is converted by all key slices; a draft tile has code of
+// its own, apart from the codes' loop, in which two slices share its keys, each for half of the rows, and masked keys
+// are left out (16 caches of 32K keys, 16 rows, 178 -> 173 us per call; 40 of 300 to 2500 60.5 -> 50.5; 512 of 50 to
+// 400 326 -> 276, 4 rows 136 -> 117).
 using Cfg8 = Cfg<1, 1, 4, 2, 3>;
 using Cfg16 = Cfg<2, 1, 4, 3, 2>;
 using Cfg16Many = Cfg<2, 1, 4, 2, 2>;
