@@ -433,7 +433,9 @@ cudaError_t launch_merge(const AttnParams& p, int sms, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, blocks <= 2 * sms ? merge_kernel<16, 2> : merge_kernel<2, 6>, p);
+  // (One cache whose units are in two pieces at most fills no batch of 16: 300 tokens, 4 rows 11.0 -> 10.9 us per call.)
+  const bool two_pieces = p.unit_ctas == 1 || p.unit_ctas == 2;
+  return cudaLaunchKernelEx(&cfg, blocks <= 2 * sms && !two_pieces ? merge_kernel<16, 2> : merge_kernel<2, 6>, p);
 }
 
 cudaError_t launch_append(AppendParams a, cudaStream_t stream) {
