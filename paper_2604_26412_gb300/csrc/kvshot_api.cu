@@ -257,7 +257,7 @@ kvshot_status check_common(const kvshot_attn_desc* d) {
         d->v_scale_exp > kMaxScaleExp)
       return KVSHOT_ERR_SHAPE;
     if (d->flags & KVSHOT_FORCE_CC) return KVSHOT_ERR_UNSUPPORTED;
-    // The tensor-memory kernel decodes fp8 tiles for stacks of up to 128 rows (not for paired blocks).
+    // Forced, the tensor-memory kernel takes fp8 stacks of up to 128 rows; the planner gives it larger ones in blocks.
     if ((d->flags & KVSHOT_FORCE_TC) && static_cast<int64_t>(d->hq / std::max(d->hkv, 1)) * d->n_query > 128)
       return KVSHOT_ERR_UNSUPPORTED;
   }
@@ -307,12 +307,13 @@ kvshot_status make_plan_for(const kvshot_attn_desc* d, bool paged, bool small_bl
   const bool tc_ok = G <= 128 && 128 % G == 0;
   // fp8 tiles: the tcgen05 kernel decodes them into f16 tiles in shared memory,
   // attn_f8.cu into MMA fragments in registers.  Up to 16 rows the latter streams the codes at
-  // 0.84-0.89 of the copy peak (4 rows: 105 us per ragged-chain call, 16 rows: 179 us per multi-layer
+  // 0.87-0.92 of the copy peak (4 rows: 102 us per ragged-chain call, 16 rows: 173 us per multi-layer
   // call, tcgen05 302 and 368 us); its MMAs pad and repeat with the rows, so from 17 rows the tcgen05
-  // kernel is ahead (hybrid tree, 32 and 48 rows: 55 and 56 us per call against 72 and 108 us).  Stacks
+  // kernel is ahead for long prefixes (16 caches of 4096 tokens, 32 and 48 rows: 59.5 and 59.3 us per call
+  // against 60.5 and 77 us).  Stacks
   // of more than 128 rows take it in 128-row blocks (the paired kernel has no fp8 form): reading the
   // codes once per block still beats the 64-row blocks of attn_f8.cu (whole hybrid tree, 256 rows:
-  // 179 us against 350 us; with the 64-row blocks of the bf16 kernel's fp8 form it was 529 us).
+  // 163 us in a graph against 350 us; with the 64-row blocks of the bf16 kernel's fp8 form it was 529 us).
   const bool fp8 = d->flags & KVSHOT_TARGET_FP8;
   const bool tc_auto = fp8 ? rows > 16 && !(small_blocks && rows > 128) : rows >= 16;
   const Kernel mma = fp8 ? Kernel::kMmaF8 : Kernel::kMma;
