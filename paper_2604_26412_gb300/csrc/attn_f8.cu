@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(CF::kThreads, CF::kMinBlocks)
 // per ragged-chain call of 64 caches against 117 us for two CTAs of three stages), 16 rows two (three would
 // spill).  48 rows take two key slices: with four, 13 warps are capped at 128 registers and spill (16 caches of 4096 tokens
 // 101 us per call, now 85).  Before this kernel the same calls took 185 us (4 rows) and 265 us (16 rows, 16 caches x 32K
-// keys, now 176 us): 64-key tiles, query rows as the MMA's M, 18.4 M instead of 13.1 M warp instructions per call of
+// keys, now 173 us): 64-key tiles, query rows as the MMA's M, 18.4 M instead of 13.1 M warp instructions per call of
 // 16 caches x 4096 tokens at 16 rows.
 // Short units are bound by what a unit costs beside its tiles.  q is converted by all key slices; a draft tile has code of
 // its own, apart from the codes' loop, in which two slices share its keys, each for half of the rows, and masked keys

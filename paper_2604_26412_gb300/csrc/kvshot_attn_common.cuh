@@ -282,8 +282,8 @@ __device__ __forceinline__ bool unit_cuts(const AttnParams& p) {
 // seq_lens[threadIdx.x], loaded early by the caller (-1: not loaded).  PK, here and below: keys
 // per prefix tile (draft tiles always hold kTileKeys).  kLaneSums: the prefix sum as one scan of the
 // lanes' sums (220 caches of 41..83 tokens, 4 rows: 58.7 -> 53.9 us per call) and not a scan per 32
-// caches, which the tcgen05 kernel of up to 128 rows keeps: it is compiled into 0.4 us less per call with it,
-// with an fp8 cache 1.3.
+// caches, which the tcgen05 kernel of up to 128 rows keeps: it is compiled into 0.3 us less per call with it
+// (16 caches x 4096), with an fp8 cache 0.5 us less at 32 query rows and 9 at 24 (85 -> 76 us).
 template <int PK = kTileKeys, int kCuts = kCutsEither, bool kLaneSums = true>
 __device__ __forceinline__ void build_plan(const AttnParams& p, int* s_len, int* s_base, int len0 = -1) {
   const int HR = p.hkv * p.row_blocks;
